@@ -269,3 +269,98 @@ def tolerance(case):
     if case["kind"] == "loss" and case["dtype"] == "f32":
         return {"rel": 2.5e-4, "max": 7e-4}
     return {"rel": 8.5e-3, "max": 0.1}
+
+
+def _exact_attention(pack, q, k, v, d_o=None):
+    """o, lse and, where d_o is given, dq, dk, dv in 64 bits: dense masked softmax attention, sample by sample."""
+    T, hq, d = q.shape
+    g = hq // k.shape[1]
+    scale = d ** -0.5
+    o, lse = torch.zeros_like(q), torch.zeros((hq, T), dtype=torch.float64, device=q.device)
+    dq, dk, dv = (torch.zeros_like(t) for t in (q, k, v))
+    for start, P, C, R in zip(pack.cu_seqlens, pack.prefix_len, pack.chosen_len, pack.rejected_len):
+        rows = slice(int(start), int(start) + int(P + C + R))
+        at = torch.arange(int(P + C + R), device=q.device)
+        hidden = (at[None, :] > at[:, None]) | ((at[:, None] >= int(P + C)) & (at[None, :] >= int(P)) & (at[None, :] < int(P + C)))
+        for h in range(hq):
+            qs, ks, vs = q[rows, h], k[rows, h // g], v[rows, h // g]
+            scores = (qs @ ks.t() * scale).masked_fill_(hidden, -math.inf)
+            lse[h, rows] = torch.logsumexp(scores, 1)
+            p = scores.sub_(lse[h, rows, None]).exp_()
+            o[rows, h] = p @ vs
+            if d_o is not None:
+                g_o = d_o[rows, h]
+                dv[rows, h // g] += p.t() @ g_o
+                ds = (g_o @ vs.t()).sub_((g_o * o[rows, h]).sum(1, keepdim=True)).mul_(p).mul_(scale)
+                dq[rows, h] = ds @ ks
+                dk[rows, h // g] += ds.t() @ qs
+    return o, lse, dq, dk, dv
+
+
+def _exact_loss(s, backward):
+    """logps and, with `backward`, loss, coef and the gradient of the logits in 64 bits."""
+    logits, n = s["logits"], s["n_segments"]
+    T, vocab = logits.shape
+    rows = torch.arange(T, device="cuda")
+    label_rows, label_targets, label_segments = (torch.cat([a, b.long()]) for a, b in (
+        (rows, s["forks"][0]), (s["targets"].long(), s["forks"][1]), (s["segments"].long(), s["forks"][2])))
+    keep = label_segments >= 0
+    label_rows, label_targets, label_segments = label_rows[keep], label_targets[keep], label_segments[keep]
+    lse = torch.cat([torch.logsumexp(logits[lo:lo + 512].double(), 1) for lo in range(0, T, 512)])
+    logps = torch.zeros(n, dtype=torch.float64, device="cuda")
+    logps.index_add_(0, label_segments, logits[label_rows, label_targets].double() - lse[label_rows])
+    if not backward:
+        return [logps]
+    x = logps.clone().requires_grad_()
+    if s["loss"] == "dpo":
+        z = x - s["reference"].double()
+        loss = -torch.nn.functional.logsigmoid(0.1 * (z[0::2] - z[1::2])).mean()
+    else:
+        mean = x / s["scored"].double()
+        if s["loss"] == "simpo":
+            loss = -torch.nn.functional.logsigmoid(2.0 * (mean[0::2] - mean[1::2]) - 0.5).mean()
+        else:
+            odds = mean - torch.log(-torch.expm1(mean))
+            loss = (-mean[0::2] - 0.1 * torch.nn.functional.logsigmoid(odds[0::2] - odds[1::2])).mean()
+    coef, = torch.autograd.grad(loss, x)
+    per_row = torch.zeros(T, dtype=torch.float64, device="cuda").index_add_(0, label_rows, coef[label_segments])
+    grad = torch.empty((T, vocab), dtype=torch.float64, device="cuda")
+    for lo in range(0, T, 512):
+        some = slice(lo, lo + 512)
+        grad[some] = (logits[some].double() - lse[some, None]).exp_().mul_(-per_row[some, None])
+    grad.index_put_((label_rows, label_targets), coef[label_segments], accumulate=True)
+    return [logps, loss.detach()[None], coef, grad]
+
+
+def _exact_layer(pack, x, w, d_out, d):
+    """out, dx and the gradients of the four weights in 64 bits."""
+    T = x.shape[0]
+    x, d_out, (wq, wk, wv, wo) = x.double(), d_out.double(), [t.double() for t in w]
+    at = np.concatenate([np.concatenate([np.arange(P + C), P + np.arange(R)])
+                         for P, C, R in zip(pack.prefix_len, pack.chosen_len, pack.rejected_len)])
+    half = torch.arange(d // 2, dtype=torch.float64, device="cuda")
+    angle = torch.as_tensor(at).double().cuda()[:, None, None] * 10000.0 ** (-2 * half / d)
+
+    def turn(t, sign):
+        cos, sin, (a, b) = angle.cos(), angle.sin() * sign, t.split(d // 2, 2)
+        return torch.cat([a * cos - b * sin, b * cos + a * sin], 2)
+
+    q, k = turn((x @ wq).view(T, -1, d), 1), turn((x @ wk).view(T, -1, d), 1)
+    o, _, dq, dk, dv = _exact_attention(pack, q, k, (x @ wv).view(T, -1, d), (d_out @ wo.t()).view(T, -1, d))
+    o, dq, dk, dv = o.view(T, -1), turn(dq, -1).view(T, -1), turn(dk, -1).view(T, -1), dv.view(T, -1)
+    dx = dq @ wq.t() + dk @ wk.t() + dv @ wv.t()
+    return [o @ wo, dx, x.t() @ dq, x.t() @ dk, x.t() @ dv, o.t() @ d_out]
+
+
+def exact(case, seed):
+    s = prepare(case, seed)
+    pack, kind = s["pack"], s["kind"]
+    if kind == "loss":
+        return _exact_loss(s, True)
+    if kind == "layer":
+        return _exact_layer(pack, s["x"], s["w"], s["d_out"], pack.head_dim)
+    q, k, v, d_o = [t.cuda().double() for t in (s["in"] if kind == "host" else (s["q"], s["k"], s["v"], s["d_o"]))]
+    if kind == "reference":
+        return [*_exact_attention(pack, q, k, v)[:2], *_exact_loss(s, False)]
+    outs = _exact_attention(pack, q, k, v, d_o)
+    return [*outs[:2], *(_exact_loss(s, True) if kind == "step" else []), *outs[2:]]
