@@ -11,7 +11,8 @@
 //                own S columns) for the second UMMA.  The two halves of a row exchange their
 //                maxima through shared memory.
 // A CTA takes two work items (query tile, query head), one after the other: items 2 b and 2 b + 1 of the list
-// (longest first; usually the same query tile and two heads of one kv head).  Barrier parities run on over both
+// (longest first; usually the same query tile and two heads of one kv head); in a launch of few items it takes one.
+// Barrier parities run on over both
 // items; the second item's Q and first K tile are requested as soon as the first item's last score product has
 // read them, i.e. they arrive while the first item's last softmax, P V and output store are still going on, and
 // the barrier initialisation, the TMEM allocation and the exit are paid once for two items.
@@ -35,6 +36,7 @@ using namespace dev;
 
 constexpr int kFwdThreads = 384;
 constexpr int kSoftmaxThreads = 256;
+constexpr int kOneItemMost = 1184;   // four items for each of the 296 CTAs that 148 SMs hold
 // Register split of the 80 per thread the launch bound allows: the first warpgroup (producer,
 // issuer) gives registers to the two softmax warpgroups.
 constexpr int kRegsWg0 = 32, kRegsSoftmax = 104;
@@ -49,6 +51,7 @@ struct FwdParams {
   int32_t* status;
   int32_t T, Hq, Hkv;
   int32_t n_items;   // query tiles x query heads
+  int32_t items_per_cta;   // 1 or 2
   float scale_log2;  // softmax_scale * log2(e)
 };
 
@@ -98,10 +101,10 @@ psa_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   volatile int* abort_flag = reinterpret_cast<volatile int*>(gen_base + L::kAbort);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // The CTA's work items: 2 b and 2 b + 1 of the list (longest first, so the CTAs stay sorted by length and the
-  // short ones still fill the tail of the launch); the last CTA of an odd count has one item.
-  const int idx0 = 2 * int(blockIdx.x), idx1 = idx0 + 1;
-  const int n_items = idx1 < prm.n_items ? 2 : 1;
+  // The CTA's work items: b of the list, or 2 b and 2 b + 1 (longest first, so the CTAs stay sorted by length and the
+  // short ones still fill the tail of the launch; the last CTA of an odd count has one item).
+  const int idx0 = prm.items_per_cta * int(blockIdx.x), idx1 = idx0 + 1;
+  const int n_items = prm.items_per_cta > 1 && idx1 < prm.n_items ? 2 : 1;
   FwdItem* s_item = reinterpret_cast<FwdItem*>(gen_base + L::kItems);
   int32_t* s_ent_all = reinterpret_cast<int32_t*>(gen_base + L::kEnt);
   const WaitCtx wctx{abort_flag, prm.status, kWaitLimitClocks};
@@ -685,7 +688,12 @@ psa_status_t launch_fwd_t(const psa_plan_t* plan, const void* q, const void* k, 
   prm.Hkv = plan->Hkv;
   prm.n_items = int32_t(plan->q_tiles.size()) * plan->Hq;
   prm.scale_log2 = plan->scale * 1.4426950408889634f;
-  const unsigned grid = unsigned(prm.n_items + 1) / 2u;   // two work items per CTA
+  // Two items per CTA pay the CTA's fixed costs once for both; one per CTA spreads a short list over more of the 296
+  // CTAs that the chip holds.  us, two -> one: 10505 tokens, 4 heads of 64 (332 items) 130 -> 65; 2954 tokens, 32 heads
+  // of 128 (768) 63 -> 53; 7965 tokens, 16 heads of 64 (1040) 56.6 -> 52.9; 5061 tokens, 32 heads of 128 (1312)
+  // 96.6 -> 100.4; 7727 tokens (2176) 79.7 -> 88.0; 31041 tokens (7904) 965 -> 1019.
+  prm.items_per_cta = prm.n_items <= kOneItemMost ? 1 : 2;
+  const unsigned grid = unsigned(prm.n_items + prm.items_per_cta - 1) / unsigned(prm.items_per_cta);
   {
     ProfileScope prof(0, stream);
     psa_fwd_kernel<D><<<grid, kFwdThreads, L::kRequest, stream>>>(tm_q, tm_k, tm_v, tm_o, prm);

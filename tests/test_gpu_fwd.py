@@ -145,3 +145,18 @@ def test_row_maximum_that_grows_from_key_tile_to_key_tile(gains):
     # the 1e-2 was stated for (measured here: 0.0106).  A wrong rescale would be off by O(1).
     raw, raw_small, excess = grad_errors(o, ro)
     assert raw_small <= 2 * TOL_O and excess <= 2 * TOL_O and max_abs(lse, rl) <= TOL_LSE, (raw, raw_small, excess, max_abs(lse, rl))
+
+
+@pytest.mark.parametrize("heads,tokens", [(4, 295), (4, 296), (5, 1184 // 5 - 1), (5, 1184 // 5 + 1)])
+def test_launches_around_the_number_of_items_at_which_a_cta_takes_two(heads, tokens):
+    # `tokens` samples of one 128-row tile at most each: heads * tokens work items (1180, 1184, 1175, 1185), odd
+    # counts among them, whose last CTA has one item.
+    pack = wl.pack_from_lengths("items", [(1 + i % 3, i % 2, 1) for i in range(tokens)], heads, heads, 64)
+    q, k, v, _ = wl.attention_inputs(pack, heads)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    o, lse = B.psa_fwd(device_plan(pack), q.cuda(), k.cuda(), v.cuda(), status=status)
+    assert read_status(status) == 0
+    ro, rl = oracle_fwd(pack, q, k, v)
+    assert max_abs(lse, rl) <= TOL_LSE
+    # rows with one to five keys: o is close to a row of v, whose bf16 rounding (|v| < 8: 2^-6) bounds the output's
+    assert max_abs(o, ro) <= 2.0 ** -6 + TOL_O
