@@ -29,7 +29,7 @@ extern "C" psa_status_t psa_fwd(const psa_plan_t* plan, const void* q, const voi
     return PSA_ERR_ALIGNMENT;
   if (!psa::plan_on_current_device(plan)) return PSA_ERR_INVALID_ARG;
   psa::note_plan_use(plan, stream);
-  return psa::launch_fwd(plan, q, k, v, o, lse, device_status, stream);
+  return psa::launch_fwd(plan, plan->whole, q, k, v, o, lse, device_status, stream);
 }
 
 extern "C" psa_status_t psa_bwd(const psa_plan_t* plan, const void* d_o, const void* q, const void* k,
@@ -45,7 +45,7 @@ extern "C" psa_status_t psa_bwd(const psa_plan_t* plan, const void* d_o, const v
     return PSA_ERR_ALIGNMENT;
   if (!psa::plan_on_current_device(plan)) return PSA_ERR_INVALID_ARG;
   psa::note_plan_use(plan, stream);
-  return psa::launch_bwd(plan, d_o, q, k, v, o, lse, dq, dk, dv, workspace, false, device_status, stream);
+  return psa::launch_bwd(plan, plan->whole, d_o, q, k, v, o, lse, dq, dk, dv, workspace, false, device_status, stream);
 }
 
 extern "C" psa_status_t psa_bwd_f32(const psa_plan_t* plan, const void* d_o, const void* q, const void* k,
@@ -61,7 +61,7 @@ extern "C" psa_status_t psa_bwd_f32(const psa_plan_t* plan, const void* d_o, con
     return PSA_ERR_ALIGNMENT;
   if (!psa::plan_on_current_device(plan)) return PSA_ERR_INVALID_ARG;
   psa::note_plan_use(plan, stream);
-  return psa::launch_bwd(plan, d_o, q, k, v, o, lse, dq, dk, dv, workspace, true, device_status, stream);
+  return psa::launch_bwd(plan, plan->whole, d_o, q, k, v, o, lse, dq, dk, dv, workspace, true, device_status, stream);
 }
 
 namespace {
@@ -111,13 +111,13 @@ extern "C" psa_status_t psa_step_host(const psa_plan_t* plan, const void* h_q, c
   if (!copy(base + a.q, h_q, nq, cudaMemcpyHostToDevice) || !copy(base + a.k, h_k, nk, cudaMemcpyHostToDevice) ||
       !copy(base + a.v, h_v, nk, cudaMemcpyHostToDevice) || !copy(base + a.d_o, h_do, nq, cudaMemcpyHostToDevice))
     return psa::check_last_cuda_error("psa_step_host copy in");
-  psa_status_t rc = psa::launch_fwd(plan, base + a.q, base + a.k, base + a.v, base + a.o,
+  psa_status_t rc = psa::launch_fwd(plan, plan->whole, base + a.q, base + a.k, base + a.v, base + a.o,
                                     reinterpret_cast<float*>(base + a.lse), device_status, stream);
   if (rc != PSA_OK) return rc;
   // o and lse are final after the forward: their copies out can leave before the backward runs.
   if (!copy(h_o, base + a.o, nq, cudaMemcpyDeviceToHost) || !copy(h_lse, base + a.lse, nl, cudaMemcpyDeviceToHost))
     return psa::check_last_cuda_error("psa_step_host copy out");
-  rc = psa::launch_bwd(plan, base + a.d_o, base + a.q, base + a.k, base + a.v, base + a.o,
+  rc = psa::launch_bwd(plan, plan->whole, base + a.d_o, base + a.q, base + a.k, base + a.v, base + a.o,
                        reinterpret_cast<const float*>(base + a.lse), base + a.dq, base + a.dk, base + a.dv,
                        base + a.ws, false, device_status, stream);
   if (rc != PSA_OK) return rc;

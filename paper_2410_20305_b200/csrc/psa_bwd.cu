@@ -5,7 +5,7 @@
 //      then, only for a pack that holds rejected rows with fewer than 32 visible keys outside
 //      their sample's first query tile (prompts shorter than 32 tokens), a small kernel that
 //      recomputes delta of those rows exactly
-//   2. main kernel: one CTA per (key tile j, kv head); it walks the query heads of the
+//   2. main kernel: one CTA per (key tile j, kv head), or a cluster of CTAs where those are few; it walks the query heads of the
 //      group and, for each, the live query tiles i of the transposed tile map.  All
 //      products are formed transposed (rows = keys) so that dK and dV accumulate in
 //      TMEM for the whole CTA lifetime and need no atomics:
@@ -89,7 +89,9 @@ enum {
 };
 
 
-template <int D>
+// kSplit: the iterations of one (key tile, kv head) are shared by the CTAs of a cluster, rank r taking the r-th
+// part of them; dV and dK are summed over the cluster through distributed shared memory before they leave.
+template <int D, bool kSplit>
 __global__ void __launch_bounds__(kBwdThreads, 1)
 psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do,
@@ -109,13 +111,21 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   float* s_delta = reinterpret_cast<float*>(smem_raw + L::kDelta);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tile_idx = prm.cta_map[2 * blockIdx.x];
-  const int hk = prm.cta_map[2 * blockIdx.x + 1];
+  uint32_t rank = 0, n_cta = 1;
+  if constexpr (kSplit) {
+    rank = cluster_ctarank();
+    n_cta = cluster_nctarank();
+  }
+  const int item = int(blockIdx.x / n_cta);
+  const int tile_idx = prm.cta_map[2 * item];
+  const int hk = prm.cta_map[2 * item + 1];
   const int g = prm.Hq / prm.Hkv;
   const TileRec rec = prm.tiles[tile_idx];
   const int32_t* ent = prm.entries + rec.list_off;
   const int n_list = rec.list_cnt;
-  const int n_it = n_list * g;
+  // Iterations of this CTA: [it0, it0 + n_it) of the n_list * g of the item (none, for some ranks of a short list).
+  const int it0 = int(uint32_t(n_list * g) * rank / n_cta);
+  const int n_it = kSplit ? int(uint32_t(n_list * g) * (rank + 1) / n_cta) - it0 : n_list * g;
   const WaitCtx wctx{abort_flag, prm.status, kWaitLimitClocks};
 
   if (threadIdx.x == 0) {
@@ -138,13 +148,14 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     for (int s = 0; s < L::kSub; ++s) tma_load_3d(sV + s * L::kSubBytes, &tm_v, s * 64, hk, rec.row0, bar(B_KV_FULL));
     tma_prefetch_desc(&tm_q);
     tma_prefetch_desc(&tm_do);
-    // ... and so are Q and dO of the first iteration (head hk * g, first entry of the list).
+    // ... and so are Q and dO of the first iteration.
     if (n_it > 0) {
-      const int qrow0 = rec.ds + (ent[0] >> 2) * kTile;
+      const int qrow0 = rec.ds + (ent[kSplit ? it0 % n_list : 0] >> 2) * kTile;
+      const int h0 = kSplit ? hk * g + it0 / n_list : hk * g;
       mbar_expect_tx(bar(B_Q_FULL0), L::kTileBytes);
-      for (int s = 0; s < L::kSub; ++s) tma_load_3d(sQ(0) + s * L::kSubBytes, &tm_q, s * 64, hk * g, qrow0, bar(B_Q_FULL0));
+      for (int s = 0; s < L::kSub; ++s) tma_load_3d(sQ(0) + s * L::kSubBytes, &tm_q, s * 64, h0, qrow0, bar(B_Q_FULL0));
       mbar_expect_tx(bar(B_DO_FULL), L::kTileBytes);
-      for (int s = 0; s < L::kSub; ++s) tma_load_3d(sDO + s * L::kSubBytes, &tm_do, s * 64, hk * g, qrow0, bar(B_DO_FULL));
+      for (int s = 0; s < L::kSub; ++s) tma_load_3d(sDO + s * L::kSubBytes, &tm_do, s * 64, h0, qrow0, bar(B_DO_FULL));
     }
     tma_prefetch_desc(&tm_dq);
   }
@@ -156,10 +167,10 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  // Iteration it -> (query head of the group, entry of the list).
-  auto head_of = [&](int it) { return hk * g + it / n_list; };
+  // Iteration it (of this CTA) -> (query head of the group, entry of the list).
+  auto head_of = [&](int it) { return hk * g + (kSplit ? it0 + it : it) / n_list; };
   auto entry_of = [&](int it) {
-    const int li = it % n_list;
+    const int li = (kSplit ? it0 + it : it) % n_list;
     return li < L::kEntCap ? s_ent[li] : ent[li];
   };
 
@@ -216,7 +227,7 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         }
         umma_commit_w(bar(B_S_FULL), issuer);
       };
-      issue_s(0);
+      if (!kSplit || n_it > 0) issue_s(0);
       for (int it = 0; it < n_it; ++it) {
         const int st = it & 1;
         // PRECISE tiles carry P^T and dS^T as two bf16 terms each.
@@ -280,6 +291,10 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     }
     __syncwarp();
   }  // warps 2, 3 of the first warpgroup are idle
+  if constexpr (kSplit) {   // the two barriers of the workers' reduction over the cluster
+    cluster_arrive(); cluster_wait();
+    cluster_arrive(); cluster_wait();
+  }
   } else if (warp < 12) {
     // ------------------------------------------------------------ workers: warps 4..11
     // Thread = one key row (TMEM lane) and one half of the 128 query columns: warps 4..7 take
@@ -311,7 +326,7 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       return x;
     };
     auto store_stat = [&](int st, float x) { (wt < 128 ? s_lse : s_delta)[st * kTile + (wt & 127)] = x; };
-    store_stat(0, load_stat(0));
+    if (!kSplit || n_it > 0) store_stat(0, load_stat(0));
     named_bar_sync(1, 256);
 
     uint32_t dse_ph = 0;  // running parity of B_DS_EMPTY
@@ -477,7 +492,83 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     tc_fence_after();
 
     // ---- epilogue: this half's columns of dV and dK (scaled) -> bf16, or fp32 as they are
-    if (prm.f32_out) {
+    if constexpr (kSplit) {
+      // CTA `owner` of the cluster writes out rows [owner * R, (owner + 1) * R) of the tile, R = 128 / n_cta.  Once
+      // every CTA has finished its products (first barrier) the tile buffers are free: each thread sends its row's
+      // half of dV and dK to the owner, which adds them to its own (second barrier).
+      const uint32_t R = uint32_t(kTile) / n_cta, owner = uint32_t(r) / R, slot_row = (uint32_t(r) % R) + R * half;
+      // receive buffer: [sender (the owner left out)][dV, dK][4-column group of a half][half x R rows] of float4
+      auto slot_addr = [&](uint32_t sender, int which, int c4) {
+        const uint32_t i = sender - (sender > owner ? 1u : 0u);
+        return base + (((i * 2 + which) * (DH / 4) + c4) * (2 * R) + slot_row) * 16u;
+      };
+      static_assert(7 * 2 * (DH / 4) * 32 * 16 <= L::kDQS, "the receive buffer of eight CTAs fits into the tile buffers");
+      __syncwarp();
+      cluster_arrive(); cluster_wait();
+      // (TMEM loads are warp-wide, while the rows of one warp may have two owners: only the rest is conditional)
+#pragma unroll
+      for (int which = 0; which < 2; ++which) {
+#pragma unroll
+        for (int ch = 0; ch < DH / 32; ++ch) {
+          uint32_t v[32];
+          tmem_ld32_wait(tmem + lane_base + (which ? kColDK : kColDV) + half * DH + ch * 32, v);
+          if (owner != rank) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const uint32_t to = cluster_map(slot_addr(rank, which, ch * 8 + i), owner);
+              if (n_it > 0) st_cluster_v4(to, v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+              else st_cluster_v4(to, 0u, 0u, 0u, 0u);
+            }
+          }
+          __syncwarp();
+        }
+      }
+      cluster_arrive(); cluster_wait();
+      const int64_t row = int64_t(rec.row0) + r;
+#pragma unroll
+      for (int which = 0; which < 2; ++which) {
+        const float mul = which ? prm.scale : 1.f;
+#pragma unroll
+        for (int ch = 0; ch < DH / 32; ++ch) {
+          uint32_t v[32];
+          tmem_ld32_wait(tmem + lane_base + (which ? kColDK : kColDV) + half * DH + ch * 32, v);
+          const int64_t at = (row * prm.Hkv + hk) * D + half * DH + ch * 32;
+          if (owner == rank && kv_valid && PSA_IN_BOUNDS(at + 31, int64_t(prm.T) * prm.Hkv * D, prm.status)) {
+            if (n_it == 0) {
+#pragma unroll
+              for (int i = 0; i < 32; ++i) v[i] = 0u;
+            }
+            for (uint32_t c = 0; c < n_cta; ++c) {
+              if (c == rank) continue;
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                const float4 a = *reinterpret_cast<const float4*>(smem_raw + (slot_addr(c, which, ch * 8 + i) - base));
+                v[4 * i + 0] = __float_as_uint(__uint_as_float(v[4 * i + 0]) + a.x);
+                v[4 * i + 1] = __float_as_uint(__uint_as_float(v[4 * i + 1]) + a.y);
+                v[4 * i + 2] = __float_as_uint(__uint_as_float(v[4 * i + 2]) + a.z);
+                v[4 * i + 3] = __float_as_uint(__uint_as_float(v[4 * i + 3]) + a.w);
+              }
+            }
+            if (prm.f32_out) {
+              float4* dst = reinterpret_cast<float4*>(static_cast<float*>(which ? prm.dk : prm.dv) + at);
+#pragma unroll
+              for (int i = 0; i < 8; ++i)
+                dst[i] = make_float4(__uint_as_float(v[4 * i + 0]) * mul, __uint_as_float(v[4 * i + 1]) * mul,
+                                     __uint_as_float(v[4 * i + 2]) * mul, __uint_as_float(v[4 * i + 3]) * mul);
+            } else {
+              uint4* dst = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(which ? prm.dk : prm.dv) + at);
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+                dst[i] = make_uint4(pack_bf16x2(__uint_as_float(v[8 * i + 0]) * mul, __uint_as_float(v[8 * i + 1]) * mul),
+                                    pack_bf16x2(__uint_as_float(v[8 * i + 2]) * mul, __uint_as_float(v[8 * i + 3]) * mul),
+                                    pack_bf16x2(__uint_as_float(v[8 * i + 4]) * mul, __uint_as_float(v[8 * i + 5]) * mul),
+                                    pack_bf16x2(__uint_as_float(v[8 * i + 6]) * mul, __uint_as_float(v[8 * i + 7]) * mul));
+            }
+          }
+          __syncwarp();
+        }
+      }
+    } else if (prm.f32_out) {
       // fp32 outputs: the accumulators leave unrounded, one row per thread.
       const int64_t row = int64_t(rec.row0) + r;
 #pragma unroll
@@ -614,6 +705,11 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     }
     if (leader) tma_wait_group_read<0>();   // shared memory must outlive the last reduce's reads (the adds
                                             // themselves complete before the kernel does)
+    if constexpr (kSplit) {   // the two barriers of the workers' reduction over the cluster
+      __syncwarp();
+      cluster_arrive(); cluster_wait();
+      cluster_arrive(); cluster_wait();
+    }
   }
 
   tc_fence_before();
@@ -629,14 +725,14 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 template <int D>
 __global__ void __launch_bounds__(256)
 psa_bwd_delta_kernel(const __nv_bfloat16* __restrict__ d_o, const __nv_bfloat16* __restrict__ o,
-                     float* __restrict__ delta, float* __restrict__ dq_accum, int64_t n_rows /* T*Hq */, int32_t T,
-                     int32_t Hq, int32_t* status) {
+                     float* __restrict__ delta, float* __restrict__ dq_accum, int64_t row0,
+                     int64_t row1 /* of T*Hq */, int32_t T, int32_t Hq, int32_t* status) {
   constexpr int kLanes = D / 8;  // threads per (t, h) row
   const int64_t gid = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int64_t row = gid / kLanes;
+  const int64_t row = row0 + gid / kLanes;
   const int part = int(gid % kLanes);
   float acc = 0.f;
-  if (row < n_rows) {
+  if (row < row1) {
     const uint4 a = reinterpret_cast<const uint4*>(d_o + row * D)[part];
     const uint4 b = reinterpret_cast<const uint4*>(o + row * D)[part];
     // the same thread clears the eight accumulator elements that belong to its eight inputs
@@ -652,7 +748,7 @@ psa_bwd_delta_kernel(const __nv_bfloat16* __restrict__ d_o, const __nv_bfloat16*
   }
 #pragma unroll
   for (int off = kLanes / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-  if (row < n_rows && part == 0) {
+  if (row < row1 && part == 0) {
     const int64_t t = row / Hq;
     const int h = int(row % Hq);
     if (PSA_IN_BOUNDS(int64_t(h) * T + t, int64_t(Hq) * T, status)) delta[int64_t(h) * T + t] = acc;
@@ -730,7 +826,7 @@ psa_bwd_convert_kernel(const float4* __restrict__ acc, uint2* __restrict__ dq, i
 }
 
 template <int D>
-psa_status_t launch_bwd_t(const psa_plan_t* plan, const void* d_o, const void* q, const void* k, const void* v,
+psa_status_t launch_bwd_t(const psa_plan_t* plan, const PlanPart& part, const void* d_o, const void* q, const void* k, const void* v,
                           const void* o, const float* lse, void* dq, void* dk, void* dv, void* workspace,
                           bool f32_out, int32_t* device_status, cudaStream_t stream) {
   using L = BwdSmem<D>;
@@ -748,26 +844,28 @@ psa_status_t launch_bwd_t(const psa_plan_t* plan, const void* d_o, const void* q
       // (with fp32 outputs dk and dv leave through per-thread stores; their maps are built but not used)
       !make_tile_map_bf16(&tm_dk, dk, T, plan->Hkv, D) || !make_tile_map_bf16(&tm_dv, dv, T, plan->Hkv, D))
     return PSA_ERR_CUDA;
-  if (cudaFuncSetAttribute(psa_bwd_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kRequest) != cudaSuccess)
+  const int split = part.bwd_split;
+  auto kernel = split > 1 ? psa_bwd_kernel<D, true> : psa_bwd_kernel<D, false>;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kRequest) != cudaSuccess)
     return PSA_ERR_CUDA;
 
-  const int64_t n_rows = T * plan->Hq;
+  const int64_t row0 = int64_t(part.row0) * plan->Hq, row1 = int64_t(part.row1) * plan->Hq, n_rows = row1 - row0;
   {
     ProfileScope prof(3, stream);
     const int64_t threads = n_rows * (D / 8);
     psa_bwd_delta_kernel<D><<<unsigned((threads + 255) / 256), 256, 0, stream>>>(
-        static_cast<const __nv_bfloat16*>(d_o), static_cast<const __nv_bfloat16*>(o), delta, dq_accum, n_rows, plan->T,
-        plan->Hq, device_status);
+        static_cast<const __nv_bfloat16*>(d_o), static_cast<const __nv_bfloat16*>(o), delta, dq_accum, row0, row1,
+        plan->T, plan->Hq, device_status);
   }
-  if (!plan->few_key_rows.empty())
-    psa_bwd_delta_few_keys_kernel<D><<<dim3(unsigned(plan->few_key_rows.size()), unsigned((plan->Hq + 3) / 4)), 128, 0, stream>>>(
-        plan->d_few_key_rows, static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k),
+  if (part.n_few > 0)
+    psa_bwd_delta_few_keys_kernel<D><<<dim3(unsigned(part.n_few), unsigned((plan->Hq + 3) / 4)), 128, 0, stream>>>(
+        plan->d_few_key_rows + part.few0, static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k),
         static_cast<const __nv_bfloat16*>(v), static_cast<const __nv_bfloat16*>(d_o), lse, delta, plan->T, plan->Hq,
         plan->Hkv, plan->scale * kLog2e, device_status);
   BwdParams prm;
   prm.tiles = plan->d_kv_tiles;
   prm.entries = plan->d_bwd_entries;
-  prm.cta_map = plan->d_bwd_cta_map;
+  prm.cta_map = plan->d_bwd_cta_map + 2 * int64_t(part.cta0);
   prm.lse = lse;
   prm.delta = delta;
   prm.dq_accum = dq_accum;
@@ -780,29 +878,39 @@ psa_status_t launch_bwd_t(const psa_plan_t* plan, const void* d_o, const void* q
   prm.Hkv = plan->Hkv;
   prm.scale = plan->scale;
   prm.scale_log2 = plan->scale * kLog2e;
-  const unsigned grid = unsigned(plan->kv_tiles.size()) * unsigned(plan->Hkv);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(unsigned(part.n_ctas) * unsigned(split));
+  cfg.blockDim = dim3(kBwdThreads);
+  cfg.dynamicSmemBytes = L::kRequest;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = unsigned(split);
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = split > 1 ? 1 : 0;
   {
     ProfileScope prof(1, stream);
-    psa_bwd_kernel<D><<<grid, kBwdThreads, L::kRequest, stream>>>(tm_q, tm_k, tm_v, tm_do, tm_dq, tm_dk, tm_dv, prm);
+    cudaLaunchKernelEx(&cfg, kernel, tm_q, tm_k, tm_v, tm_do, tm_dq, tm_dk, tm_dv, prm);
   }
   if (!f32_out) {
     ProfileScope prof(4, stream);
     const int64_t n_vec4 = n_rows * D / 4;
     psa_bwd_convert_kernel<<<unsigned((n_vec4 + 1023) / 1024), 256, 0, stream>>>(
-        reinterpret_cast<const float4*>(dq_accum), static_cast<uint2*>(dq), n_vec4);
+        reinterpret_cast<const float4*>(dq_accum) + row0 * D / 4, static_cast<uint2*>(dq) + row0 * D / 4, n_vec4);
   }
   return check_last_cuda_error("psa_bwd launch");
 }
 
 }  // namespace
 
-psa_status_t launch_bwd(const psa_plan_t* plan, const void* d_o, const void* q, const void* k, const void* v,
+psa_status_t launch_bwd(const psa_plan_t* plan, const PlanPart& part, const void* d_o, const void* q, const void* k, const void* v,
                         const void* o, const float* lse, void* dq, void* dk, void* dv, void* workspace,
                         bool f32_out, int32_t* device_status, void* stream) {
   if (plan->d == 128)
-    return launch_bwd_t<128>(plan, d_o, q, k, v, o, lse, dq, dk, dv, workspace, f32_out, device_status,
+    return launch_bwd_t<128>(plan, part, d_o, q, k, v, o, lse, dq, dk, dv, workspace, f32_out, device_status,
                              cudaStream_t(stream));
-  return launch_bwd_t<64>(plan, d_o, q, k, v, o, lse, dq, dk, dv, workspace, f32_out, device_status,
+  return launch_bwd_t<64>(plan, part, d_o, q, k, v, o, lse, dq, dk, dv, workspace, f32_out, device_status,
                           cudaStream_t(stream));
 }
 

@@ -70,5 +70,5 @@ extern "C" psa_status_t psa_bwd_static_scratch(const psa_plan_t* plan, const voi
   // launch_bwd clears the dq accumulator itself (it must start at zero) and overwrites delta,
   // so whatever the previous call left in the array does not matter.
   psa::note_plan_use(plan, stream);
-  return psa::launch_bwd(plan, d_o, q, k, v, o, lse, dq, dk, dv, scratch, false, device_status, stream);
+  return psa::launch_bwd(plan, plan->whole, d_o, q, k, v, o, lse, dq, dk, dv, scratch, false, device_status, stream);
 }

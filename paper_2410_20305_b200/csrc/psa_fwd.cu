@@ -668,7 +668,7 @@ psa_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 }
 
 template <int D>
-psa_status_t launch_fwd_t(const psa_plan_t* plan, const void* q, const void* k, const void* v, void* o, float* lse,
+psa_status_t launch_fwd_t(const psa_plan_t* plan, const PlanPart& part, const void* q, const void* k, const void* v, void* o, float* lse,
                           int32_t* device_status, cudaStream_t stream) {
   using L = FwdSmem<D>;
   CUtensorMap tm_q, tm_k, tm_v, tm_o;
@@ -678,7 +678,7 @@ psa_status_t launch_fwd_t(const psa_plan_t* plan, const void* q, const void* k, 
   if (cudaFuncSetAttribute(psa_fwd_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kRequest) != cudaSuccess)
     return PSA_ERR_CUDA;
   FwdParams prm;
-  prm.tiles = plan->d_q_tiles;
+  prm.tiles = plan->d_q_tiles + part.q_tile0;
   prm.entries = plan->d_fwd_entries;
   prm.o = static_cast<__nv_bfloat16*>(o);
   prm.lse = lse;
@@ -686,7 +686,7 @@ psa_status_t launch_fwd_t(const psa_plan_t* plan, const void* q, const void* k, 
   prm.T = plan->T;
   prm.Hq = plan->Hq;
   prm.Hkv = plan->Hkv;
-  prm.n_items = int32_t(plan->q_tiles.size()) * plan->Hq;
+  prm.n_items = part.n_q_tiles * plan->Hq;
   prm.scale_log2 = plan->scale * 1.4426950408889634f;
   // Two items per CTA pay the CTA's fixed costs once for both; one per CTA spreads a short list over more of the 296
   // CTAs that the chip holds.  us, two -> one: 10505 tokens, 4 heads of 64 (332 items) 130 -> 65; 2954 tokens, 32 heads
@@ -703,10 +703,10 @@ psa_status_t launch_fwd_t(const psa_plan_t* plan, const void* q, const void* k, 
 
 }  // namespace
 
-psa_status_t launch_fwd(const psa_plan_t* plan, const void* q, const void* k, const void* v, void* o, float* lse,
+psa_status_t launch_fwd(const psa_plan_t* plan, const PlanPart& part, const void* q, const void* k, const void* v, void* o, float* lse,
                         int32_t* device_status, void* stream) {
-  if (plan->d == 128) return launch_fwd_t<128>(plan, q, k, v, o, lse, device_status, cudaStream_t(stream));
-  return launch_fwd_t<64>(plan, q, k, v, o, lse, device_status, cudaStream_t(stream));
+  if (plan->d == 128) return launch_fwd_t<128>(plan, part, q, k, v, o, lse, device_status, cudaStream_t(stream));
+  return launch_fwd_t<64>(plan, part, q, k, v, o, lse, device_status, cudaStream_t(stream));
 }
 
 }  // namespace psa

@@ -36,6 +36,15 @@ struct FewKeyRow {
 };
 static_assert(sizeof(FewKeyRow) == 16, "FewKeyRow is 4 int32");
 
+// The part of a plan that one launch covers.  Offsets index the plan's device arrays.
+struct PlanPart {
+  int32_t row0 = 0, row1 = 0;            // packed rows
+  int32_t q_tile0 = 0, n_q_tiles = 0;    // query tiles
+  int32_t cta0 = 0, n_ctas = 0;          // (key tile, kv head) pairs of the backward's launch order
+  int32_t few0 = 0, n_few = 0;           // few-key rows
+  int32_t bwd_split = 1;                 // CTAs (a cluster) that share the iterations of one such pair: 1, 2, 4 or 8
+};
+
 }  // namespace psa
 
 struct psa_plan {
@@ -47,6 +56,7 @@ struct psa_plan {
   std::vector<int32_t> fwd_entries, bwd_entries;
   // Launch order of the backward CTAs: pairs (index into kv_tiles, kv head).
   std::vector<int32_t> bwd_cta_map;
+  psa::PlanPart whole;
   std::vector<psa::FewKeyRow> few_key_rows;
   // device copy (one allocation, taken from and returned to a small process-wide cache so that a
   // plan per step costs no cudaMalloc / cudaFree and no host synchronisation)
@@ -96,9 +106,9 @@ struct BwdWorkspace {
 };
 BwdWorkspace bwd_workspace_layout(int64_t T, int Hq, int d);
 
-psa_status_t launch_fwd(const psa_plan_t* plan, const void* q, const void* k, const void* v, void* o,
+psa_status_t launch_fwd(const psa_plan_t* plan, const PlanPart& part, const void* q, const void* k, const void* v, void* o,
                         float* lse, int32_t* device_status, void* stream);
-psa_status_t launch_bwd(const psa_plan_t* plan, const void* d_o, const void* q, const void* k,
+psa_status_t launch_bwd(const psa_plan_t* plan, const PlanPart& part, const void* d_o, const void* q, const void* k,
                         const void* v, const void* o, const float* lse, void* dq, void* dk, void* dv,
                         void* workspace, bool f32_out, int32_t* device_status, void* stream);
 }  // namespace psa

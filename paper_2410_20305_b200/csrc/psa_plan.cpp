@@ -13,7 +13,6 @@
 #include <mutex>
 #include <new>
 #include <numeric>
-#include <queue>
 #include <utility>
 #include <vector>
 
@@ -62,6 +61,95 @@ bool precise_rows(int i, int len, int cs, int rs) {
   const int q0 = i * kTile, q1 = std::min(q0 + kTile, len);
   const int q = std::max(q0, rs);                   // first rejected row of the tile, if any
   return q < q1 && cs + (q - rs + 1) < kTile;       // it sees the prompt and q - rs + 1 own keys
+}
+
+// Launch order of the backward for the samples [s0, s1), appended to the plan's list, and the number of CTAs that share
+// the iterations of one (key tile, kv head) pair.
+//
+// Order: every CTA adds its dQ contributions into the fp32 accumulator rows of its sample and query-head group, so CTAs
+// that share those rows are launched together: the rows then stay in L2 while they are being updated.  Samples with
+// the most work first, then kv head, then the sample's key tiles, longest list first.  That can leave a ragged tail
+// (its makespan over 148 SMs is 8 % above the mean on the Llama-3-8B-shaped pack).  Alternative: hand out the last 30 %
+// of the work longest first.  That evens out the finish but gives up the L2 locality of the tail, so it is taken only
+// when a list-scheduling simulation says it shortens the makespan by more than 5 %.
+void order_backward(psa_plan_t* p, const std::vector<std::vector<int32_t>>& tiles_of, int s0, int s1, int n_sm,
+                    PlanPart* part) {
+  typedef std::vector<std::pair<int32_t, int32_t>> Order;   // (key tile record, kv head)
+  std::vector<int64_t> work(s1 - s0, 0);
+  for (int s = s0; s < s1; ++s)
+    for (int32_t t : tiles_of[s]) work[s - s0] += p->kv_tiles[t].list_cnt;
+  std::vector<int> order(s1 - s0);
+  std::iota(order.begin(), order.end(), s0);
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return work[a - s0] > work[b - s0]; });
+  Order ctas;
+  int64_t total_work = 0;
+  for (int s : order)
+    for (int hk = 0; hk < p->Hkv; ++hk)
+      for (int32_t t : tiles_of[s]) {
+        ctas.emplace_back(t, hk);
+        total_work += p->kv_tiles[t].list_cnt;
+      }
+  // Makespan of an order on `slots` slots, a pair with a list of n taking cost(n).
+  std::vector<int64_t> free_at;
+  auto makespan = [&](const Order& o, size_t slots, auto cost) {
+    int64_t end = 0;
+    if (o.size() <= slots) {
+      for (const auto& c : o) end = std::max(end, cost(p->kv_tiles[c.first].list_cnt));
+      return end;
+    }
+    free_at.assign(slots, 0);   // a heap, earliest first: the earliest slot takes the pair and sinks to its new place
+    for (const auto& c : o) {
+      const int64_t t = free_at[0] + cost(p->kv_tiles[c.first].list_cnt);
+      end = std::max(end, t);
+      size_t i = 0;
+      for (size_t k = 1; k < slots; k = 2 * i + 1) {
+        if (k + 1 < slots && free_at[k + 1] < free_at[k]) ++k;
+        if (free_at[k] >= t) break;
+        free_at[i] = free_at[k];
+        i = k;
+      }
+      free_at[i] = t;
+    }
+    return end;
+  };
+  Order hybrid = ctas;
+  int64_t acc = 0;
+  size_t at = 0;
+  while (at < hybrid.size() && acc * 10 < total_work * 7) acc += p->kv_tiles[hybrid[at++].first].list_cnt;
+  std::stable_sort(hybrid.begin() + at, hybrid.end(), [&](const auto& a, const auto& b) {
+    return p->kv_tiles[a.first].list_cnt > p->kv_tiles[b.first].list_cnt;
+  });
+  auto length = [](int32_t n) { return int64_t(n); };
+  if (makespan(ctas, n_sm, length) * 100 > makespan(hybrid, n_sm, length) * 105) ctas.swap(hybrid);
+  // CTAs per pair: where the pairs are few, the longest of them lasts longer than the rest of the chip is busy.  Sharing
+  // a pair costs each of its CTAs the fixed part of a CTA and the reduction over the cluster, so it only pays below two
+  // pairs per SM.  Of 148 SMs clusters of 2, 4 and 8 reach 148, 132 and 120.  us of the whole backward, split 1 / 2 / 4 / 8:
+  //   436 tokens, 8/2 heads of 128 (8 pairs)        53 / 37 / 25 / 24     1814 tokens, 8/2 of 64 (34)      62 / 38 / 26 / 40
+  //   3160 tokens, 8/2 heads of 64 (50)             261 / 108 / 59 / 82   11799 tokens, 8/2 of 128 (186)   818 / 645 / 660 / 794
+  //   16700 tokens, 8/2 heads of 128 (262)          1383 / 1262 / 1374 / 1482
+  //   5061 tokens, 32/8 heads of 128 (328)          264 / 270 / 354 / 575
+  if (ctas.size() <= 2 * size_t(n_sm)) {
+    const int64_t iter_ns = p->d == 128 ? 2050 : 1600, fixed_ns = p->d == 128 ? 8000 : 7000, combine_ns = 3000;
+    const int64_t group = p->Hq / p->Hkv;
+    int64_t best = makespan(ctas, n_sm, [&](int32_t n) { return n * group * iter_ns + fixed_ns; });
+    for (int split : {2, 4, 8}) {
+      const size_t slots = split == 2 ? n_sm / 2 : (split == 4 ? n_sm * 33 / 148 : n_sm * 15 / 148);
+      const int64_t t = makespan(ctas, std::max<size_t>(slots, 1), [&](int32_t n) {
+        return (n * group + split - 1) / split * iter_ns + fixed_ns + combine_ns;
+      });
+      if (t * 100 < best * 95) {
+        best = t;
+        part->bwd_split = split;
+      }
+    }
+  }
+  part->cta0 = int32_t(p->bwd_cta_map.size() / 2);
+  part->n_ctas = int32_t(ctas.size());
+  p->bwd_cta_map.reserve(p->bwd_cta_map.size() + ctas.size() * 2);
+  for (const auto& c : ctas) {
+    p->bwd_cta_map.push_back(c.first);
+    p->bwd_cta_map.push_back(c.second);
+  }
 }
 
 }  // namespace
@@ -153,72 +241,27 @@ extern "C" psa_status_t psa_plan(const int32_t* cu_seqlens, const int32_t* prefi
   std::stable_sort(p->q_tiles.begin(), p->q_tiles.end(), longest_first);
   std::stable_sort(p->kv_tiles.begin(), p->kv_tiles.end(), longest_first);
   p->bwd_workspace_bytes = psa::bwd_workspace_layout(p->T, p->Hq, p->d).total;
-  // Backward CTA order.  Every CTA adds its dQ contributions into the fp32 accumulator rows of
-  // its sample and query-head group, so CTAs that share those rows are launched together: the
-  // rows then stay in L2 while they are being updated.  Samples with the most work first, then
-  // kv head, then the sample's key tiles, longest list first.
   {
-    std::vector<int64_t> work(n_samples, 0);
+    int n_sm = 148;
+    if (!(flags & PSA_PLAN_HOST_ONLY)) {
+      int dev = 0, v = 0;
+      if (cudaGetDevice(&dev) == cudaSuccess &&
+          cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
+        n_sm = v;
+    }
+    // Key tiles of every sample, longest list first.
     std::vector<std::vector<int32_t>> tiles_of(n_samples);
-    std::vector<int32_t> sample_of_start(n_samples);
     for (size_t t = 0; t < p->kv_tiles.size(); ++t) {
       // the sample is found from its start row (cu_seqlens is increasing over non-empty samples)
       const int32_t ds = p->kv_tiles[t].ds;
       int s = int(std::upper_bound(cu_seqlens, cu_seqlens + n_samples + 1, ds) - cu_seqlens) - 1;
       while (s + 1 < n_samples && cu_seqlens[s + 1] == ds) ++s;   // skip zero-length samples
-      work[s] += p->kv_tiles[t].list_cnt;
-      tiles_of[s].push_back(int32_t(t));                          // already longest first
+      tiles_of[s].push_back(int32_t(t));
     }
-    std::vector<int> order(n_samples);
-    std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return work[a] > work[b]; });
-    std::vector<std::pair<int32_t, int32_t>> ctas;   // (key tile record, kv head)
-    ctas.reserve(p->kv_tiles.size() * n_kv_heads);
-    int64_t total_work = 0;
-    for (int s : order)
-      for (int hk = 0; hk < n_kv_heads; ++hk)
-        for (int32_t t : tiles_of[s]) {
-          ctas.emplace_back(t, hk);
-          total_work += p->kv_tiles[t].list_cnt;
-        }
-    // The grouped order can leave a ragged tail (its makespan over 148 SMs is 8 % above the mean
-    // on the Llama-3-8B-shaped pack).  Alternative: hand out the last 30 % of the work longest
-    // first.  That evens out the finish but gives up the L2 locality of the tail, so it is taken
-    // only when a list-scheduling simulation says it shortens the makespan by more than 5 %.
-    {
-      int n_sm = 148;
-      if (!(flags & PSA_PLAN_HOST_ONLY)) {
-        int dev = 0, v = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-          n_sm = v;
-      }
-      auto makespan = [&](const std::vector<std::pair<int32_t, int32_t>>& order_) {
-        std::priority_queue<int64_t, std::vector<int64_t>, std::greater<int64_t>> sm;
-        for (int i = 0; i < n_sm; ++i) sm.push(0);
-        int64_t end = 0;
-        for (const auto& c : order_) {
-          const int64_t t = sm.top() + p->kv_tiles[c.first].list_cnt;
-          sm.pop();
-          sm.push(t);
-          end = std::max(end, t);
-        }
-        return end;
-      };
-      std::vector<std::pair<int32_t, int32_t>> hybrid = ctas;
-      int64_t acc = 0;
-      size_t split = 0;
-      while (split < hybrid.size() && acc * 10 < total_work * 7) acc += p->kv_tiles[hybrid[split++].first].list_cnt;
-      std::stable_sort(hybrid.begin() + split, hybrid.end(), [&](const auto& a, const auto& b) {
-        return p->kv_tiles[a.first].list_cnt > p->kv_tiles[b.first].list_cnt;
-      });
-      if (makespan(ctas) * 100 > makespan(hybrid) * 105) ctas.swap(hybrid);
-    }
-    p->bwd_cta_map.reserve(ctas.size() * 2);
-    for (const auto& c : ctas) {
-      p->bwd_cta_map.push_back(c.first);
-      p->bwd_cta_map.push_back(c.second);
-    }
+    p->whole.row1 = p->T;
+    p->whole.n_q_tiles = int32_t(p->q_tiles.size());
+    p->whole.n_few = int32_t(p->few_key_rows.size());
+    psa::order_backward(p, tiles_of, 0, n_samples, n_sm, &p->whole);
   }
 
   if (!(flags & PSA_PLAN_HOST_ONLY)) {
