@@ -256,10 +256,13 @@ psa_status_t psa_bwd_static_scratch(const psa_plan_t* plan, const void* d_o, con
 
 /*
  * psa_step_host -- one forward and one backward pass of the attention (Algorithm 3; the
- * two calls above) on HOST buffers.  The call enqueues on `stream`, in this order: the
- * copies of q, k, v, d_o from host memory into the arena, psa_fwd, psa_bwd, and the copies
- * of o, lse, dq, dk, dv back to host memory.  It does not synchronise: the outputs are valid
- * once the stream has reached the end of the call's work.  Calls on different streams with
+ * two calls above) on HOST buffers.  The call enqueues the copies of q, k, v, d_o from host
+ * memory into the arena, psa_fwd, psa_bwd, and the copies of o, lse, dq, dk, dv back to host
+ * memory; a larger pack goes in parts (runs of samples), whose copies in and out run on two
+ * streams of the library under the kernels of other parts.  All of it starts behind what
+ * `stream` holds at the call, and `stream` ends behind all of it; a call on a capturing stream
+ * uses that stream alone.  It does not synchronise: the outputs are valid once the stream has
+ * reached the end of the call's work.  Calls on different streams with
  * different arenas overlap (one call's copies with another's kernels).
  *   h_q, h_do   host bf16 [T, Hq, d]       h_k, h_v    host bf16 [T, Hkv, d]      (in)
  *   h_o, h_dq   host bf16 [T, Hq, d]       h_dk, h_dv  host bf16 [T, Hkv, d]      (out)

@@ -36,7 +36,8 @@ struct FewKeyRow {
 };
 static_assert(sizeof(FewKeyRow) == 16, "FewKeyRow is 4 int32");
 
-// The part of a plan that one launch covers.  Offsets index the plan's device arrays.
+// The part of a plan that one launch covers: the whole pack, or a run of whole samples of it (psa_step_host overlaps
+// the copies of one run with the kernels of another).  Offsets index the plan's device arrays.
 struct PlanPart {
   int32_t row0 = 0, row1 = 0;            // packed rows
   int32_t q_tile0 = 0, n_q_tiles = 0;    // query tiles
@@ -52,11 +53,15 @@ struct psa_plan {
   float scale = 0.f;
   int64_t useful_pairs = 0, live_tiles = 0, partial_tiles = 0;
   size_t bwd_workspace_bytes = 0;
-  std::vector<psa::TileRec> q_tiles, kv_tiles;   // sorted, longest list first
+  std::vector<psa::TileRec> q_tiles, kv_tiles;   // sorted, longest list first (within the pack, then within each part)
   std::vector<int32_t> fwd_entries, bwd_entries;
   // Launch order of the backward CTAs: pairs (index into kv_tiles, kv head).
   std::vector<int32_t> bwd_cta_map;
   psa::PlanPart whole;
+  // Runs of whole samples for psa_step_host (none for a pack that is not worth splitting).  Where there are several,
+  // their query tiles and CTA pairs follow those of the whole pack in q_tiles and bwd_cta_map, in the order of the runs.
+  std::vector<psa::PlanPart> parts;
+  mutable void* host_pipe = nullptr;   // psa::HostPipe of psa_step_host, created by its first call
   std::vector<psa::FewKeyRow> few_key_rows;
   // device copy (one allocation, taken from and returned to a small process-wide cache so that a
   // plan per step costs no cudaMalloc / cudaFree and no host synchronisation)
@@ -105,6 +110,9 @@ struct BwdWorkspace {
   size_t total;
 };
 BwdWorkspace bwd_workspace_layout(int64_t T, int Hq, int d);
+
+// Hands the streams and events of psa_step_host back to their process-wide pool.
+void give_host_pipe(void* pipe);
 
 psa_status_t launch_fwd(const psa_plan_t* plan, const PlanPart& part, const void* q, const void* k, const void* v, void* o,
                         float* lse, int32_t* device_status, void* stream);

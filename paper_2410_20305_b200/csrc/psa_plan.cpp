@@ -112,15 +112,17 @@ void order_backward(psa_plan_t* p, const std::vector<std::vector<int32_t>>& tile
     }
     return end;
   };
-  Order hybrid = ctas;
-  int64_t acc = 0;
-  size_t at = 0;
-  while (at < hybrid.size() && acc * 10 < total_work * 7) acc += p->kv_tiles[hybrid[at++].first].list_cnt;
-  std::stable_sort(hybrid.begin() + at, hybrid.end(), [&](const auto& a, const auto& b) {
-    return p->kv_tiles[a.first].list_cnt > p->kv_tiles[b.first].list_cnt;
-  });
-  auto length = [](int32_t n) { return int64_t(n); };
-  if (makespan(ctas, n_sm, length) * 100 > makespan(hybrid, n_sm, length) * 105) ctas.swap(hybrid);
+  if (part == &p->whole) {
+    Order hybrid = ctas;
+    int64_t acc = 0;
+    size_t at = 0;
+    while (at < hybrid.size() && acc * 10 < total_work * 7) acc += p->kv_tiles[hybrid[at++].first].list_cnt;
+    std::stable_sort(hybrid.begin() + at, hybrid.end(), [&](const auto& a, const auto& b) {
+      return p->kv_tiles[a.first].list_cnt > p->kv_tiles[b.first].list_cnt;
+    });
+    auto length = [](int32_t n) { return int64_t(n); };
+    if (makespan(ctas, n_sm, length) * 100 > makespan(hybrid, n_sm, length) * 105) ctas.swap(hybrid);
+  }
   // CTAs per pair: where the pairs are few, the longest of them lasts longer than the rest of the chip is busy.  Sharing
   // a pair costs each of its CTAs the fixed part of a CTA and the reduction over the cluster, so it only pays below two
   // pairs per SM.  Of 148 SMs clusters of 2, 4 and 8 reach 148, 132 and 120.  us of the whole backward, split 1 / 2 / 4 / 8:
@@ -128,7 +130,9 @@ void order_backward(psa_plan_t* p, const std::vector<std::vector<int32_t>>& tile
   //   3160 tokens, 8/2 heads of 64 (50)             261 / 108 / 59 / 82   11799 tokens, 8/2 of 128 (186)   818 / 645 / 660 / 794
   //   16700 tokens, 8/2 heads of 128 (262)          1383 / 1262 / 1374 / 1482
   //   5061 tokens, 32/8 heads of 128 (328)          264 / 270 / 354 / 575
-  if (ctas.size() <= 2 * size_t(n_sm)) {
+  if (part != &p->whole) {   // (a part runs under the copies of another: no simulation, only what fits at once)
+    while (part->bwd_split < 4 && ctas.size() * part->bwd_split * 2 <= size_t(n_sm) * 33 / 37) part->bwd_split *= 2;
+  } else if (ctas.size() <= 2 * size_t(n_sm)) {
     const int64_t iter_ns = p->d == 128 ? 2050 : 1600, fixed_ns = p->d == 128 ? 8000 : 7000, combine_ns = 3000;
     const int64_t group = p->Hq / p->Hkv;
     int64_t best = makespan(ctas, n_sm, [&](int32_t n) { return n * group * iter_ns + fixed_ns; });
@@ -262,6 +266,37 @@ extern "C" psa_status_t psa_plan(const int32_t* cu_seqlens, const int32_t* prefi
     p->whole.n_q_tiles = int32_t(p->q_tiles.size());
     p->whole.n_few = int32_t(p->few_key_rows.size());
     psa::order_backward(p, tiles_of, 0, n_samples, n_sm, &p->whole);
+
+    // Parts for psa_step_host: runs of whole samples of about a sixth of the pack (4 to 24 differ by 5 %; with more
+    // parts the copies get too short for the link) and of at least 2 MB of q, which the link takes 40 us for.  A
+    // smaller pack has none: its copies take less time than the overlap costs the host.
+    const int64_t row_bytes = int64_t(p->Hq) * p->d * 2, least_bytes = int64_t(2) << 20;
+    const int64_t least = std::max(int64_t(p->T) / 6, (least_bytes + row_bytes - 1) / row_bytes);
+    std::vector<int> first{0};   // first sample of each part
+    for (int s = 0; s < n_samples; ++s)
+      if (cu_seqlens[s + 1] - cu_seqlens[first.back()] >= least || s + 1 == n_samples) first.push_back(s + 1);
+    if (first.size() > 2) {
+      const size_t n_whole = p->q_tiles.size();
+      for (size_t i = 0; i + 1 < first.size(); ++i) {
+        psa::PlanPart w;
+        w.row0 = cu_seqlens[first[i]];
+        w.row1 = cu_seqlens[first[i + 1]];
+        if (w.row1 == w.row0) continue;
+        w.q_tile0 = int32_t(p->q_tiles.size());
+        for (size_t t = 0; t < n_whole; ++t) {   // (still longest list first)
+          const TileRec r = p->q_tiles[t];
+          if (r.row0 >= w.row0 && r.row0 < w.row1) p->q_tiles.push_back(r);
+        }
+        w.n_q_tiles = int32_t(p->q_tiles.size()) - w.q_tile0;
+        const int32_t n_few = int32_t(p->few_key_rows.size());
+        while (w.few0 < n_few && p->few_key_rows[w.few0].row < w.row0) ++w.few0;
+        while (w.few0 + w.n_few < n_few && p->few_key_rows[w.few0 + w.n_few].row < w.row1) ++w.n_few;
+        psa::order_backward(p, tiles_of, first[i], first[i + 1], n_sm, &w);
+        p->parts.push_back(w);
+      }
+    } else if (int64_t(p->T) * row_bytes >= least_bytes) {
+      p->parts.push_back(p->whole);
+    }
   }
 
   if (!(flags & PSA_PLAN_HOST_ONLY)) {
@@ -437,6 +472,7 @@ extern "C" psa_status_t psa_plan_destroy(psa_plan_t* p) {
     if (cur >= 0 && cur != p->device) cudaSetDevice(cur);
     give_entry(e);
   }
+  if (p->host_pipe) psa::give_host_pipe(p->host_pipe);
   delete p;
   return st;
 }
@@ -456,9 +492,8 @@ extern "C" psa_status_t psa_plan_stats(const psa_plan_t* p, int64_t* total_token
 extern "C" psa_status_t psa_plan_counts(const psa_plan_t* p, int32_t direction, int32_t* n_tiles,
                                         int32_t* n_entries) {
   if (!p || (direction != 0 && direction != 1)) return PSA_ERR_INVALID_ARG;
-  const auto& tiles = direction ? p->kv_tiles : p->q_tiles;
   const auto& entries = direction ? p->bwd_entries : p->fwd_entries;
-  if (n_tiles) *n_tiles = int32_t(tiles.size());
+  if (n_tiles) *n_tiles = direction ? int32_t(p->kv_tiles.size()) : p->whole.n_q_tiles;
   if (n_entries) *n_entries = int32_t(entries.size());
   return PSA_OK;
 }
@@ -468,7 +503,8 @@ extern "C" psa_status_t psa_plan_export(const psa_plan_t* p, int32_t direction, 
   if (!p || (direction != 0 && direction != 1) || !tiles || !entries) return PSA_ERR_INVALID_ARG;
   const auto& t = direction ? p->kv_tiles : p->q_tiles;
   const auto& e = direction ? p->bwd_entries : p->fwd_entries;
-  if (!t.empty()) std::memcpy(tiles, t.data(), t.size() * sizeof(TileRec));
+  const size_t n = direction ? t.size() : size_t(p->whole.n_q_tiles);
+  if (n) std::memcpy(tiles, t.data(), n * sizeof(TileRec));
   if (!e.empty()) std::memcpy(entries, e.data(), e.size() * sizeof(int32_t));
   return PSA_OK;
 }

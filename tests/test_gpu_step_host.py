@@ -65,3 +65,37 @@ def test_step_host_rejects_small_arena_and_null():
     with pytest.raises(B.PsaError) as e:
         B.psa_step_host(plan, q, k, v, d_o, *outs, small)
     assert e.value.code == 1
+
+
+@pytest.mark.parametrize("lengths,heads", [
+    ([(90, 40, 55), (0, 30, 29), (200, 129, 127), (0, 0, 1), (64, 64, 64), (5, 300, 20), (2, 150, 190)] * 2, (32, 8, 64)),
+    ([(700, 80, 90)], (32, 8, 128)),             # one sample: one part
+    ([(1, 1, 0), (1400, 30, 40), (3, 0, 2)], (16, 16, 128))])
+def test_step_host_in_parts_equals_the_device_calls(lengths, heads):
+    # packs of more than 2 MB of q go in parts; two calls in a row on two streams share the plan's copy streams
+    pack = wl.pack_from_lengths("parts", lengths, *heads)
+    assert pack.total_tokens * heads[0] * heads[2] * 2 > 2 << 20
+    plan = device_plan(pack)
+    sets = []
+    for seed in (7, 8):
+        t = [x.pin_memory() for x in wl.attention_inputs(pack, seed)]
+        q, k = t[0], t[1]
+        out = [torch.zeros_like(q).pin_memory(), torch.zeros((heads[0], pack.total_tokens)).pin_memory(),
+               torch.zeros_like(q).pin_memory(), torch.zeros_like(k).pin_memory(), torch.zeros_like(k).pin_memory()]
+        sets.append((t, out, torch.empty(B.psa_step_host_arena_bytes(plan), dtype=torch.uint8, device="cuda"),
+                     torch.cuda.Stream()))
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    for t, out, arena, stream in sets:
+        B.psa_step_host(plan, *t, *out, arena, status=status, stream=stream.cuda_stream)
+    for t, out, arena, stream in sets:
+        stream.synchronize()
+    assert read_status(status) == 0
+    for t, out, arena, stream in sets:
+        q, k, v, d_o = (x.cuda() for x in t)
+        o, lse = B.psa_fwd(plan, q, k, v)
+        grads = B.psa_bwd(plan, d_o, q, k, v, o, lse)
+        assert torch.equal(out[0], o.cpu()) and torch.equal(out[1], lse.cpu())
+        for got, want in zip(out[2:], grads):   # sums of fp32 adds in another order, rounded to bf16
+            want = want.cpu().double()
+            assert ((got.double() - want).abs() <= 2.0 ** -7 * want.abs() + 1e-4).all()
