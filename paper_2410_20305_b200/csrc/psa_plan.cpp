@@ -128,7 +128,8 @@ void order_backward(psa_plan_t* p, const std::vector<std::vector<int32_t>>& tile
   // pairs per SM.  Of 148 SMs clusters of 2, 4 and 8 reach 148, 132 and 120.  us of the whole backward, split 1 / 2 / 4 / 8:
   //   436 tokens, 8/2 heads of 128 (8 pairs)        53 / 37 / 25 / 24     1814 tokens, 8/2 of 64 (34)      62 / 38 / 26 / 40
   //   3160 tokens, 8/2 heads of 64 (50)             261 / 108 / 59 / 82   11799 tokens, 8/2 of 128 (186)   818 / 645 / 660 / 794
-  //   16700 tokens, 8/2 heads of 128 (262)          1383 / 1262 / 1374 / 1482
+  //   16700 tokens, 8/2 heads of 128 (262)          1383 / 1262 / 1374 / 1482 in short runs, 1376 / 1389 in long ones,
+  //   where the power limit sets the clock: a prediction of less than 10 % is not worth it.
   //   5061 tokens, 32/8 heads of 128 (328)          264 / 270 / 354 / 575
   if (part != &p->whole) {   // (a part runs under the copies of another: no simulation, only what fits at once)
     while (part->bwd_split < 4 && ctas.size() * part->bwd_split * 2 <= size_t(n_sm) * 33 / 37) part->bwd_split *= 2;
@@ -141,7 +142,7 @@ void order_backward(psa_plan_t* p, const std::vector<std::vector<int32_t>>& tile
       const int64_t t = makespan(ctas, std::max<size_t>(slots, 1), [&](int32_t n) {
         return (n * group + split - 1) / split * iter_ns + fixed_ns + combine_ns;
       });
-      if (t * 100 < best * 95) {
+      if (t * 100 < best * 90) {
         best = t;
         part->bwd_split = split;
       }
