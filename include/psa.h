@@ -312,6 +312,18 @@ psa_status_t dpo_logp(const void* logits, int32_t logits_dtype, int64_t n_rows, 
                       float* out, int32_t* device_status, void* stream);
 
 /*
+ * dpo_logp_f64sum -- dpo_logp with the sums of the responses taken in fp64 and rounded once.
+ *   scratch   device memory of 8 * (n_segments + 1) bytes, 8-byte aligned; contents on entry are
+ *             ignored, on exit undefined
+ * Everything else, and the errors, as dpo_logp.
+ */
+psa_status_t dpo_logp_f64sum(const void* logits, int32_t logits_dtype, int64_t n_rows, int64_t vocab,
+                             int64_t row_stride, const int32_t* targets, const int32_t* segment_ids,
+                             const int32_t* fork_rows, const int32_t* fork_targets,
+                             const int32_t* fork_segments, int32_t n_forks, int32_t n_segments,
+                             float* out, void* scratch, int32_t* device_status, void* stream);
+
+/*
  * psa_position_ids -- position ids of the shared layout (Section 3.1: the positions are set so
  * that the sequences are the same as in the paired format): prompt and chosen tokens count on
  * from 0 at the sample start, the j-th rejected token gets P + j.  Host only.

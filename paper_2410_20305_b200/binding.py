@@ -27,7 +27,7 @@ EXPORTED_SYMBOLS = (
     "psa_bwd_static_scratch", "dpo_loss", "dpo_logp_bwd", "psa_pack_ffd", "psa_position_ids", "psa_rope",
     "psa_step_host_arena_bytes", "psa_step_host", "simpo_loss", "orpo_loss", "psa_bwd_f32",
     "psa_check_device_status", "psa_selftest_wait_expiry", "psa_logp_labels", "psa_pack_ffd_emit",
-    "psa_selftest_bounds",
+    "psa_selftest_bounds", "dpo_logp_f64sum",
 )
 
 
@@ -84,6 +84,7 @@ def load_library():
     lib.psa_rope.argtypes = [vp, vp, vp, i64, i32, i32, f32, vp]
     lib.dpo_logp_bwd.argtypes = [vp, i32, i64, i64, i64, vp, vp, vp, vp, vp, i32, i32, vp, vp, vp, vp]
     lib.dpo_logp.argtypes = [vp, i32, i64, i64, i64, vp, vp, vp, vp, vp, i32, i32, vp, vp, vp]
+    lib.dpo_logp_f64sum.argtypes = [vp, i32, i64, i64, i64, vp, vp, vp, vp, vp, i32, i32, vp, vp, vp, vp]
     for name in EXPORTED_SYMBOLS:
         if name == "psa_step_host_arena_bytes":
             lib.psa_step_host_arena_bytes.restype = C.c_size_t
@@ -304,10 +305,11 @@ def dpo_logp(logits, targets, segment_ids, n_segments, fork_rows=None, fork_targ
         fork_rows = fork_targets = fork_segments = None
     if out is None:
         out = torch.empty(n_segments, dtype=torch.float32, device=logits.device)
-    _check("dpo_logp", load_library().dpo_logp(_ptr(logits), dt, n_rows, vocab, logits.stride(0) if n_rows > 1 else vocab,
-                                               _ptr(targets), _ptr(segment_ids), _ptr(fork_rows), _ptr(fork_targets),
-                                               _ptr(fork_segments), n_forks, n_segments, _ptr(out), _ptr(status),
-                                               _stream(stream)))
+    scratch = torch.empty(n_segments + 1, dtype=torch.float64, device=logits.device)
+    _check("dpo_logp", load_library().dpo_logp_f64sum(
+        _ptr(logits), dt, n_rows, vocab, logits.stride(0) if n_rows > 1 else vocab, _ptr(targets), _ptr(segment_ids),
+        _ptr(fork_rows), _ptr(fork_targets), _ptr(fork_segments), n_forks, n_segments, _ptr(out), _ptr(scratch),
+        _ptr(status), _stream(stream)))
     return out
 
 

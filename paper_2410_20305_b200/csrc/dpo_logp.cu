@@ -3,7 +3,9 @@
 // live logits row exactly once with 16-byte coalesced loads, keeps a running
 // (max, sum of exp) per thread in fp32, merges across the warp with shuffles and
 // across warps through shared memory, and adds  logit[target] - lse  into
-// out[segment] with one atomic per scored label.
+// out[segment] with one atomic per scored label, or, where the caller gives scratch for them, into
+// fp64 sums that the last CTA to finish rounds into out: a response of 250 tokens is then off by its
+// lse's and one final rounding (3e-8) instead of 250 (1e-7 to 4e-7).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -78,15 +80,31 @@ __global__ void __launch_bounds__(kLogpThreads)
 dpo_logp_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_stride, const int32_t* __restrict__ targets,
                 const int32_t* __restrict__ segment_ids, const int32_t* __restrict__ fork_rows,
                 const int32_t* __restrict__ fork_targets, const int32_t* __restrict__ fork_segments, int32_t n_forks,
-                int32_t n_segments, float* __restrict__ out, int32_t* __restrict__ status) {
+                int32_t n_segments, float* __restrict__ out, double* __restrict__ sums /* [n_segments], or null */,
+                uint32_t* __restrict__ n_done, int32_t* __restrict__ status) {
   constexpr int E = Vec<T>::kElems;
   const int64_t row = blockIdx.x;
   const int32_t seg = segment_ids[row];
-  // Which labels does this row score?  (At most a handful of forks exist per pack.)
-  int32_t fork = -1;
-  for (int f = 0; f < n_forks; ++f)
-    if (fork_rows[f] == row) fork = f;  // block-uniform
-  if (seg < 0 && fork < 0) return;     // dead row: its logits are never read
+  // Every warp looks through the whole fork list, one entry per lane: the answer is block-uniform.
+  bool forked = false;
+  for (int f = threadIdx.x & 31; f < n_forks; f += 32) forked |= fork_rows[f] == row;
+  forked = __any_sync(0xffffffffu, forked);
+  // With fp64 sums every CTA counts itself when it has added its own; the last one rounds them all.
+  auto finish = [&]() {   // by one warp
+    if (!sums) return;
+    uint32_t before = 0;
+    if ((threadIdx.x & 31) == 0) {
+      __threadfence();
+      before = atomicAdd(n_done, 1u);
+      __threadfence();
+    }
+    if (__shfl_sync(0xffffffffu, before, 0) != gridDim.x - 1) return;
+    for (int g = threadIdx.x & 31; g < n_segments; g += 32) out[g] = float(__ldcg(sums + g));
+  };
+  if (seg < 0 && !forked) {            // dead row: its logits are never read
+    if (threadIdx.x < 32) finish();
+    return;
+  }
 
   const T* x = logits + row * row_stride;
   const uint4* xv = reinterpret_cast<const uint4*>(x);
@@ -118,10 +136,19 @@ dpo_logp_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_stride,
     acc.s = s;
   }
   for (; i < n_vec; i += kLogpThreads) {
-    float y[E];
+    float y[E];   // (one vector at a time, as above: 12180 x 2429 bf16, whose rows are all remainder, 22.6 -> 21.6 us)
     Vec<T>::unpack(ld_stream(xv + i), y);
+    float mx = y[0];
 #pragma unroll
-    for (int j = 0; j < E; ++j) acc.merge(y[j] * kLog2e, 1.f);
+    for (int j = 1; j < E; ++j) mx = fmaxf(mx, y[j]);
+    mx *= kLog2e;
+    const float mn = fmaxf(acc.m, mx);
+    const float sh = (mn == -INFINITY) ? 0.f : mn;
+    float s = acc.s * ex2_approx(acc.m - sh);
+#pragma unroll
+    for (int j = 0; j < E; ++j) s += ex2_approx(fmaf(y[j], kLog2e, -sh));
+    acc.m = mn;
+    acc.s = s;
   }
   for (int64_t j = n_vec * E + threadIdx.x; j < vocab; j += kLogpThreads)  // ragged tail of the row
     acc.merge(Vec<T>::load1(x + j) * kLog2e, 1.f);
@@ -152,26 +179,29 @@ dpo_logp_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_stride,
         if (g < 0) return;
         if (g >= n_segments) { if (status) atomicOr(status, PSA_DEVSTAT_BAD_SEGMENT); return; }
         if (y < 0 || y >= vocab) { if (status) atomicOr(status, PSA_DEVSTAT_BAD_TARGET); return; }
-        atomicAdd(out + g, Vec<T>::load1(x + y) - lse);
+        if (sums) atomicAdd(sums + g, double(Vec<T>::load1(x + y)) - double(lse));
+        else atomicAdd(out + g, Vec<T>::load1(x + y) - lse);
       };
       score(targets[row], seg);
-      if (fork >= 0) {
+      if (forked) {
         // Several forks may name the same row only if the caller built them so; score each.
         for (int f = 0; f < n_forks; ++f)
           if (fork_rows[f] == row) score(fork_targets[f], fork_segments[f]);
       }
     }
+    __syncwarp();
+    finish();
   }
 }
 
 }  // namespace
 }  // namespace psa
 
-extern "C" psa_status_t dpo_logp(const void* logits, int32_t logits_dtype, int64_t n_rows, int64_t vocab,
-                                 int64_t row_stride, const int32_t* targets, const int32_t* segment_ids,
-                                 const int32_t* fork_rows, const int32_t* fork_targets,
-                                 const int32_t* fork_segments, int32_t n_forks, int32_t n_segments, float* out,
-                                 int32_t* device_status, void* stream) {
+namespace {
+psa_status_t run_logp(const void* logits, int32_t logits_dtype, int64_t n_rows, int64_t vocab, int64_t row_stride,
+                      const int32_t* targets, const int32_t* segment_ids, const int32_t* fork_rows,
+                      const int32_t* fork_targets, const int32_t* fork_segments, int32_t n_forks, int32_t n_segments,
+                      float* out, double* sums, int32_t* device_status, void* stream) {
   if (n_rows < 0 || vocab <= 0 || row_stride < vocab || n_forks < 0 || n_segments < 0) return PSA_ERR_INVALID_ARG;
   if (n_segments > 0 && !out) return PSA_ERR_INVALID_ARG;
   if (n_rows > 0 && (!logits || !targets || !segment_ids)) return PSA_ERR_INVALID_ARG;
@@ -182,18 +212,44 @@ extern "C" psa_status_t dpo_logp(const void* logits, int32_t logits_dtype, int64
   // the stride is not used when there is a single row
   if ((reinterpret_cast<uintptr_t>(logits) & 15) || (n_rows > 1 && ((row_stride * esz) & 15))) return PSA_ERR_ALIGNMENT;
   cudaStream_t st = cudaStream_t(stream);
-  if (n_segments > 0 && cudaMemsetAsync(out, 0, sizeof(float) * size_t(n_segments), st) != cudaSuccess)
+  if (n_rows == 0) sums = nullptr;   // nothing runs that would round them
+  if (sums) {
+    if (cudaMemsetAsync(sums, 0, sizeof(double) * (size_t(n_segments) + 1), st) != cudaSuccess) return PSA_ERR_CUDA;
+  } else if (n_segments > 0 && cudaMemsetAsync(out, 0, sizeof(float) * size_t(n_segments), st) != cudaSuccess) {
     return PSA_ERR_CUDA;
+  }
   if (n_rows == 0) return PSA_OK;
+  uint32_t* n_done = sums ? reinterpret_cast<uint32_t*>(sums + n_segments) : nullptr;
   const unsigned grid = unsigned(n_rows);
   psa::ProfileScope prof(2, stream);
   if (logits_dtype == PSA_DTYPE_F32)
     psa::dpo_logp_kernel<float, 4><<<grid, psa::kLogpThreads, 0, st>>>(
         static_cast<const float*>(logits), vocab, row_stride, targets, segment_ids, fork_rows, fork_targets,
-        fork_segments, n_forks, n_segments, out, device_status);
+        fork_segments, n_forks, n_segments, out, sums, n_done, device_status);
   else
     psa::dpo_logp_kernel<__nv_bfloat16, 4><<<grid, psa::kLogpThreads, 0, st>>>(
         static_cast<const __nv_bfloat16*>(logits), vocab, row_stride, targets, segment_ids, fork_rows, fork_targets,
-        fork_segments, n_forks, n_segments, out, device_status);
+        fork_segments, n_forks, n_segments, out, sums, n_done, device_status);
   return psa::check_last_cuda_error("dpo_logp launch");
+}
+}  // namespace
+
+extern "C" psa_status_t dpo_logp(const void* logits, int32_t logits_dtype, int64_t n_rows, int64_t vocab,
+                                 int64_t row_stride, const int32_t* targets, const int32_t* segment_ids,
+                                 const int32_t* fork_rows, const int32_t* fork_targets,
+                                 const int32_t* fork_segments, int32_t n_forks, int32_t n_segments, float* out,
+                                 int32_t* device_status, void* stream) {
+  return run_logp(logits, logits_dtype, n_rows, vocab, row_stride, targets, segment_ids, fork_rows, fork_targets,
+                  fork_segments, n_forks, n_segments, out, nullptr, device_status, stream);
+}
+
+extern "C" psa_status_t dpo_logp_f64sum(const void* logits, int32_t logits_dtype, int64_t n_rows, int64_t vocab,
+                                        int64_t row_stride, const int32_t* targets, const int32_t* segment_ids,
+                                        const int32_t* fork_rows, const int32_t* fork_targets,
+                                        const int32_t* fork_segments, int32_t n_forks, int32_t n_segments, float* out,
+                                        void* scratch, int32_t* device_status, void* stream) {
+  if (!scratch) return PSA_ERR_INVALID_ARG;
+  if (reinterpret_cast<uintptr_t>(scratch) & 7) return PSA_ERR_ALIGNMENT;
+  return run_logp(logits, logits_dtype, n_rows, vocab, row_stride, targets, segment_ids, fork_rows, fork_targets,
+                  fork_segments, n_forks, n_segments, out, static_cast<double*>(scratch), device_status, stream);
 }

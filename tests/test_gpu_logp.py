@@ -125,3 +125,19 @@ def test_rows_that_begin_with_a_block_of_minus_infinity(dtype):
     ref = orc.dpo_logp_grad(wl.to_f64(x), tok.numpy(), seg, coef.cpu().double().numpy())
     assert np.isfinite(grad).all()
     assert np.abs(grad - ref).max() <= (2e-6 if dtype == torch.float32 else 2.0 ** -8)
+
+
+@pytest.mark.parametrize("dtype,vocab,rows", [(torch.float32, 3, 4000), (torch.bfloat16, 515, 3000), (torch.bfloat16, 4096 + 8, 1500)])
+def test_long_responses_are_summed_without_the_rounding_of_a_running_sum(dtype, vocab, rows):
+    x, _ = wl.logits_and_tokens(rows, (vocab + 7) // 8 * 8, 31, 3.0 ** 0.5, dtype)
+    rng = np.random.default_rng(4)
+    targets = rng.integers(0, vocab, rows).astype(np.int32)
+    seg = np.where(np.arange(rows) % 7 == 0, -1, np.arange(rows) * 3 // rows).astype(np.int32)
+    dev = lambda a: torch.as_tensor(a).cuda()  # noqa: E731
+    xd = x.cuda()[:, :vocab]
+    got = B.dpo_logp(xd, dev(targets), dev(seg), 4, dev(np.array([0, 7], np.int32)), dev(np.array([1, 2], np.int32)),
+                     dev(np.array([0, 2], np.int32))).cpu().double().numpy()
+    want = orc.dpo_logp(wl.to_f64(x)[:, :vocab], targets, seg, 4, [0, 7], [1, 2], [0, 2])
+    # per row half an ulp of its fp32 log-sum-exp (below 16: 5e-7) and the exponentials' error of the same size, with
+    # signs that differ from row to row; then one rounding of the sum (6e-8 of it)
+    assert got[3] == 0 and (np.abs(got - want) <= 1e-6 * 4 * np.sqrt(rows) + 6e-8 * np.abs(want)).all()
