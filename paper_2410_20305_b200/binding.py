@@ -101,18 +101,24 @@ def _check(fn, code):
 
 
 def _i32(a):
+    if type(a) is np.ndarray and a.dtype == np.int32 and a.flags.c_contiguous:
+        return a
     return np.ascontiguousarray(np.asarray(a, dtype=np.int32))
 
 
+# Pointers and streams are handed over as plain integers (every such argument is declared c_void_p).
 def _stream(stream):
     if stream is not None:
-        return C.c_void_p(int(stream))
+        return int(stream)
     import torch
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream) if torch.cuda.is_available() else C.c_void_p(0)
+    if not torch.cuda.is_initialized() and not torch.cuda.is_available():
+        return 0
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)   # the handle without the 3 us of a Stream object
+    return raw(torch.cuda.current_device()) if raw else torch.cuda.current_stream().cuda_stream
 
 
 def _ptr(t):
-    return C.c_void_p(0) if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _want(t, name, shape, dtype, cuda=True, placement=True):
@@ -136,6 +142,15 @@ def _want_attention(plan, bf16, f32=(), lse=None, cuda=True):
     import torch
     T, d = plan.total_tokens, plan.head_dim
     heads = {"q": plan.n_q_heads, "kv": plan.n_kv_heads}
+    # One look at tensors that are as they have to be; what is wrong, and the order in which that is said, below.
+    fits = lse is None or (lse.dtype == torch.float32 and lse.shape == (plan.n_q_heads, T) and lse.is_contiguous()
+                           and lse.is_cuda == cuda)
+    shape = {kind: (T, n, d) for kind, n in heads.items()}
+    for dtype, group in ((torch.bfloat16, bf16), (torch.float32, f32)):
+        for _, t, kind in group:
+            fits = fits and (t.dtype == dtype and t.shape == shape[kind] and t.is_contiguous() and t.is_cuda == cuda)
+    if fits:
+        return
     for placement in (False, True):
         for name, t, kind in bf16:
             _want(t, name, (T, heads[kind], d), torch.bfloat16, cuda, placement)
