@@ -48,5 +48,7 @@ class AttentionLayer:
         B.psa_rope(dq, self.neg, self.theta, out=dq)
         B.psa_rope(dk, self.neg, self.theta, out=dk)
         dq2, dk2, dv2 = dq.view(T, -1), dk.view(T, -1), dv.view(T, -1)
-        dx = dq2 @ wq.t() + dk2 @ wk.t() + dv2 @ wv.t()
+        # one sum for the three products: two additions of [T, hidden] matrices and two roundings less
+        dx = dq2 @ wq.t()
+        dx.addmm_(dk2, wk.t()).addmm_(dv2, wv.t())
         return dx, x.t() @ dq2, x.t() @ dk2, x.t() @ dv2, dwo
