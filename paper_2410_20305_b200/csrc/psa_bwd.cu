@@ -56,6 +56,7 @@ struct BwdParams {
   void* dv;
   int32_t* status;
   int32_t T, Hq, Hkv;
+  int32_t row_end;          // end of the part: lse and delta past it are not read
   int32_t f32_out;          // gradients leave as fp32: dk, dv from the accumulators, dq = dq_accum
   float scale, scale_log2;
 };
@@ -319,7 +320,7 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     auto load_stat = [&](int it) {
       const int64_t qrow = int64_t(rec.ds) + (entry_of(it) >> 2) * kTile + (wt & 127);
       float x = 0.f;
-      if (qrow < prm.T && PSA_IN_BOUNDS(int64_t(head_of(it)) * prm.T + qrow, int64_t(prm.Hq) * prm.T, prm.status)) {
+      if (qrow < prm.row_end && PSA_IN_BOUNDS(int64_t(head_of(it)) * prm.T + qrow, int64_t(prm.Hq) * prm.T, prm.status)) {
         const int64_t idx = int64_t(head_of(it)) * prm.T + qrow;
         x = wt < 128 ? prm.lse[idx] * kLog2e : prm.delta[idx];
       }
@@ -838,11 +839,13 @@ psa_status_t launch_bwd_t(const psa_plan_t* plan, const PlanPart& part, const vo
   float* delta = reinterpret_cast<float*>(wsp + ws.delta_off);
 
   CUtensorMap tm_q, tm_k, tm_v, tm_do, tm_dq, tm_dk, tm_dv;
-  if (!make_tile_map_bf16(&tm_q, q, T, plan->Hq, D) || !make_tile_map_bf16(&tm_k, k, T, plan->Hkv, D) ||
-      !make_tile_map_bf16(&tm_v, v, T, plan->Hkv, D) || !make_tile_map_bf16(&tm_do, d_o, T, plan->Hq, D) ||
-      !make_tile_map(&tm_dq, dq_accum, T, plan->Hq, D, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, 32, 128) ||
+  // The maps end with the part: a ragged last tile reads zeros past it, never rows that may not have arrived yet.
+  const int64_t rows = part.row1;
+  if (!make_tile_map_bf16(&tm_q, q, rows, plan->Hq, D) || !make_tile_map_bf16(&tm_k, k, rows, plan->Hkv, D) ||
+      !make_tile_map_bf16(&tm_v, v, rows, plan->Hkv, D) || !make_tile_map_bf16(&tm_do, d_o, rows, plan->Hq, D) ||
+      !make_tile_map(&tm_dq, dq_accum, rows, plan->Hq, D, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, 32, 128) ||
       // (with fp32 outputs dk and dv leave through per-thread stores; their maps are built but not used)
-      !make_tile_map_bf16(&tm_dk, dk, T, plan->Hkv, D) || !make_tile_map_bf16(&tm_dv, dv, T, plan->Hkv, D))
+      !make_tile_map_bf16(&tm_dk, dk, rows, plan->Hkv, D) || !make_tile_map_bf16(&tm_dv, dv, rows, plan->Hkv, D))
     return PSA_ERR_CUDA;
   const int split = part.bwd_split;
   auto kernel = split > 1 ? psa_bwd_kernel<D, true> : psa_bwd_kernel<D, false>;
@@ -874,6 +877,7 @@ psa_status_t launch_bwd_t(const psa_plan_t* plan, const PlanPart& part, const vo
   prm.f32_out = f32_out ? 1 : 0;
   prm.status = device_status;
   prm.T = plan->T;
+  prm.row_end = part.row1;
   prm.Hq = plan->Hq;
   prm.Hkv = plan->Hkv;
   prm.scale = plan->scale;

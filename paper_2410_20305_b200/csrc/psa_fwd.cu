@@ -672,8 +672,10 @@ psa_status_t launch_fwd_t(const psa_plan_t* plan, const PlanPart& part, const vo
                           int32_t* device_status, cudaStream_t stream) {
   using L = FwdSmem<D>;
   CUtensorMap tm_q, tm_k, tm_v, tm_o;
-  if (!make_tile_map_bf16(&tm_q, q, plan->T, plan->Hq, D) || !make_tile_map_bf16(&tm_k, k, plan->T, plan->Hkv, D) ||
-      !make_tile_map_bf16(&tm_v, v, plan->T, plan->Hkv, D) || !make_tile_map_bf16(&tm_o, o, plan->T, plan->Hq, D))
+  // The maps end with the part: a ragged last tile reads zeros past it, never rows that may not have arrived yet.
+  const int64_t rows = part.row1;
+  if (!make_tile_map_bf16(&tm_q, q, rows, plan->Hq, D) || !make_tile_map_bf16(&tm_k, k, rows, plan->Hkv, D) ||
+      !make_tile_map_bf16(&tm_v, v, rows, plan->Hkv, D) || !make_tile_map_bf16(&tm_o, o, rows, plan->Hq, D))
     return PSA_ERR_CUDA;
   if (cudaFuncSetAttribute(psa_fwd_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kRequest) != cudaSuccess)
     return PSA_ERR_CUDA;

@@ -82,8 +82,8 @@ def test_step_host_in_parts_equals_the_device_calls(lengths, heads):
         q, k = t[0], t[1]
         out = [torch.zeros_like(q).pin_memory(), torch.zeros((heads[0], pack.total_tokens)).pin_memory(),
                torch.zeros_like(q).pin_memory(), torch.zeros_like(k).pin_memory(), torch.zeros_like(k).pin_memory()]
-        sets.append((t, out, torch.empty(B.psa_step_host_arena_bytes(plan), dtype=torch.uint8, device="cuda"),
-                     torch.cuda.Stream()))
+        sets.append((t, out, torch.full((B.psa_step_host_arena_bytes(plan),), 0xff, dtype=torch.uint8, device="cuda"),
+                     torch.cuda.Stream()))   # (0xff: every float in it is NaN)
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
     torch.cuda.synchronize()
     for t, out, arena, stream in sets:
