@@ -267,10 +267,10 @@ __device__ __forceinline__ float block_lse2(MaxSum acc, float2* s_part /* [kThre
 // kStaged: the row is kept in shared memory between the sweeps, brought in by bulk copies in kParts pieces (the first
 // sweep starts on the first piece).  Many small CTAs per SM keep loads, exponentials and stores of different rows
 // in flight at the same time.
-// Otherwise the second sweep reads the row again, from L2: at two CTAs of 1024 threads per SM 296 rows are between
-// their sweeps, loaded with an evict-last policy in the first and evict-first in the second.
-template <typename T, int kThreads, bool kStaged>
-__global__ void __launch_bounds__(kThreads, kStaged ? 1536 / kThreads : 2048 / kThreads)
+// Otherwise the second sweep reads the row again, from L2: with kPerSm CTAs of 1024 threads per SM, 148 kPerSm rows are
+// between their sweeps, loaded with an evict-last policy in the first and evict-first in the second.
+template <typename T, int kThreads, bool kStaged, int kPerSm>
+__global__ void __launch_bounds__(kThreads, kPerSm)
 dpo_logp_bwd_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_stride, const int32_t* __restrict__ targets,
                     const int32_t* __restrict__ segment_ids, const int32_t* __restrict__ fork_rows,
                     const int32_t* __restrict__ fork_targets, const int32_t* __restrict__ fork_segments,
@@ -354,22 +354,26 @@ dpo_logp_bwd_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_str
 // Row size -> kernel (us of the whole call, 2/3 of the rows live; before: 1024 threads, one CTA per SM, two sweeps):
 //   up to 32 KB   staged, 128 threads      12180 x 2429 bf16 172 -> 27, 8000 x 8192 bf16 152 -> 38
 //   up to 96 KB   staged, 256 threads      2048 x 32000 bf16 68 -> 41 (128 threads: 44; two sweeps: 46 to 52)
-//   longer        two sweeps, 1024 threads 16215 x 128256 bf16 1325 -> 1238 (5.6 TB/s of one read of the live rows and
-//                 one write), 4096 x 32000 fp32 184 -> 150 (staged: 175)
+//   up to 320 KB  two sweeps, two CTAs per SM   16215 x 128256 bf16 1325 -> 1238 (5.6 TB/s of one read of the live rows
+//                 and one write), 4096 x 32000 fp32 184 -> 150 (staged: 175)
+//   longer        two sweeps, one CTA per SM    3312 x 115288 fp32, 360 rows live: 264 as before (two per SM: 297, their
+//                 296 rows of 461 KB are more than L2 holds)
 // Clusters of 2 to 8 CTAs that share a staged row were slower (1538 and more on 16215 x 128256: barriers, and too few
 // rows in flight), and so was, over the range, a persistent CTA that streams rows through a ring of bulk copies (1197
 // there, but 265 against 247 on 4096 x 50257 fp32 and 94 against 86 on 1000 x 128256 bf16).
-constexpr int64_t kStagedSmall = 32 * 1024, kStagedMost = 96 * 1024;
+constexpr int64_t kStagedSmall = 32 * 1024, kStagedMost = 96 * 1024, kTwoPerSmMost = 320 * 1024;
 
-template <typename T, int kThreads, bool kStaged>
+template <typename T, int kThreads, bool kStaged, int kPerSm>
 psa_status_t launch_logp_bwd(const T* logits, int64_t n_rows, int64_t vocab, int64_t row_stride, const int32_t* targets,
                              const int32_t* segment_ids, const int32_t* fork_rows, const int32_t* fork_targets,
                              const int32_t* fork_segments, int32_t n_forks, int32_t n_segments, const float* coef,
                              T* dlogits, int32_t* status, cudaStream_t stream) {
-  auto kernel = dpo_logp_bwd_kernel<T, kThreads, kStaged>;
-  const size_t smem = kStaged ? size_t(vocab / Elem<T>::kVec) * 16 : 0;
-  if (smem > 40 * 1024 &&
-      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kStagedMost)) != cudaSuccess)
+  auto kernel = dpo_logp_bwd_kernel<T, kThreads, kStaged, kPerSm>;
+  // (one CTA per SM: more than half of the SM's shared memory keeps a second one out)
+  constexpr size_t kAlone = 120 * 1024;
+  const size_t smem = kStaged ? size_t(vocab / Elem<T>::kVec) * 16 : (kPerSm == 1 ? kAlone : 0);
+  if (smem > 40 * 1024 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               int(kPerSm == 1 ? kAlone : size_t(kStagedMost))) != cudaSuccess)
     return PSA_ERR_CUDA;
   kernel<<<unsigned(n_rows), kThreads, smem, stream>>>(logits, vocab, row_stride, targets, segment_ids, fork_rows,
                                                       fork_targets, fork_segments, n_forks, n_segments, coef, dlogits,
@@ -380,9 +384,10 @@ psa_status_t launch_logp_bwd(const T* logits, int64_t n_rows, int64_t vocab, int
 template <typename T, typename... Args>
 psa_status_t dispatch_logp_bwd(const T* logits, int64_t n_rows, int64_t vocab, Args... args) {
   const int64_t bytes = vocab / Elem<T>::kVec * 16;
-  if (bytes <= kStagedSmall) return launch_logp_bwd<T, 128, true>(logits, n_rows, vocab, args...);
-  if (bytes <= kStagedMost) return launch_logp_bwd<T, 256, true>(logits, n_rows, vocab, args...);
-  return launch_logp_bwd<T, 1024, false>(logits, n_rows, vocab, args...);
+  if (bytes <= kStagedSmall) return launch_logp_bwd<T, 128, true, 12>(logits, n_rows, vocab, args...);
+  if (bytes <= kStagedMost) return launch_logp_bwd<T, 256, true, 6>(logits, n_rows, vocab, args...);
+  if (bytes <= kTwoPerSmMost) return launch_logp_bwd<T, 1024, false, 2>(logits, n_rows, vocab, args...);
+  return launch_logp_bwd<T, 1024, false, 1>(logits, n_rows, vocab, args...);
 }
 
 }  // namespace

@@ -1,4 +1,4 @@
-"""dpo_logp_bwd at the row sizes where it changes its kernel (rows up to 32 KB, up to 96 KB, longer), with ragged
+"""dpo_logp_bwd at the row sizes where it changes its kernel (rows up to 32, 96 and 320 KB, longer), with ragged
 ends, rows shorter than one 16-byte vector, labels on the first and the last element, and -inf logits."""
 import numpy as np
 import pytest
@@ -12,8 +12,8 @@ from gpu_util import read_status
 
 pytestmark = pytest.mark.gpu
 
-BF16 = (5, 1031, 16384, 16392 + 5, 49152, 49160 + 3, 70001)      # 32 KB = 16384, 96 KB = 49152
-F32 = (3, 515, 8192, 8196 + 1, 24576, 24580 + 3, 40001)          # 32 KB = 8192, 96 KB = 24576
+BF16 = (5, 1031, 16384, 16392 + 5, 49152, 49160 + 3, 163840, 163849)      # 32 KB = 16384, 96 KB = 49152, 320 KB = 163840
+F32 = (3, 515, 8192, 8196 + 1, 24576, 24580 + 3, 81920, 81925)          # 32 KB = 8192, 96 KB = 24576, 320 KB = 81920
 
 
 @pytest.mark.parametrize("dtype,vocab", [(torch.bfloat16, v) for v in BF16] + [(torch.float32, v) for v in F32])
