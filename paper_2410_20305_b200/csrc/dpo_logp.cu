@@ -4,9 +4,7 @@
 // (max, sum of exp) per thread in fp32, merges across the warp with shuffles and
 // across warps through shared memory, and adds  logit[target] - lse  into
 // out[segment] with one atomic per scored label, or, where the caller gives scratch for them, into
-// fp64 sums that the last live row's CTA to finish rounds into out (a first kernel clears the sums
-// and counts the live rows; counting every row in the main kernel cost its dead rows, which have
-// nothing else to do, 3 % of the whole forward at 15154 rows, 1200 of them live): a response of 250 tokens is then off by its
+// fp64 sums that are rounded into out at the end: a response of 250 tokens is then off by its
 // lse's and one final rounding (3e-8) instead of 250 (1e-7 to 4e-7).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -105,13 +103,23 @@ dpo_logp_start_kernel(const int32_t* __restrict__ segment_ids, int64_t n_rows, c
   if (threadIdx.x == 0) *n_left = s_live;
 }
 
+__global__ void dpo_logp_round_kernel(const double* __restrict__ sums, float* __restrict__ out, int32_t n_segments) {
+  const int32_t g = blockIdx.x * blockDim.x + threadIdx.x;
+  if (g < n_segments) out[g] = float(sums[g]);
+}
+
+// Logits up to this size let the last live row round the fp64 sums; above, a kernel of its own does.  The wait of
+// every row's CTA for its place in the count costs 3.5 % of the kernel (16215 x 128256 bf16 265 -> 274 us, 4096 x 50257
+// fp32 107 -> 111) and the count of the live rows 4 us more; the extra launch costs 2 us, and the host as much.
+constexpr int64_t kCountBytes = int64_t(128) << 20;
+
 template <typename T, int kUnroll>
 __global__ void __launch_bounds__(kLogpThreads)
 dpo_logp_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_stride, const int32_t* __restrict__ targets,
                 const int32_t* __restrict__ segment_ids, const int32_t* __restrict__ fork_rows,
                 const int32_t* __restrict__ fork_targets, const int32_t* __restrict__ fork_segments, int32_t n_forks,
                 int32_t n_segments, float* __restrict__ out, double* __restrict__ sums /* [n_segments], or null */,
-                uint32_t* __restrict__ n_left /* live rows not finished */, int32_t* __restrict__ status) {
+                uint32_t* __restrict__ n_left /* live rows not finished, or null */, int32_t* __restrict__ status) {
   constexpr int E = Vec<T>::kElems;
   const int64_t row = blockIdx.x;
   const int32_t seg = segment_ids[row];
@@ -119,9 +127,10 @@ dpo_logp_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_stride,
   bool forked = false;
   for (int f = threadIdx.x & 31; f < n_forks; f += 32) forked |= fork_rows[f] == row;
   forked = __any_sync(0xffffffffu, forked);
-  // With fp64 sums every live row counts itself when it has added its own; the last one rounds them all.
+  // In a small launch with fp64 sums every live row counts itself when it has added its own; the last one rounds them
+  // all.
   auto finish = [&]() {   // by one warp
-    if (!sums) return;
+    if (!n_left) return;
     uint32_t before = 0;
     if ((threadIdx.x & 31) == 0) {
       __threadfence();
@@ -240,8 +249,12 @@ psa_status_t run_logp(const void* logits, int32_t logits_dtype, int64_t n_rows, 
   if ((reinterpret_cast<uintptr_t>(logits) & 15) || (n_rows > 1 && ((row_stride * esz) & 15))) return PSA_ERR_ALIGNMENT;
   cudaStream_t st = cudaStream_t(stream);
   if (n_rows == 0) sums = nullptr;   // nothing runs that would round them
-  uint32_t* n_left = sums ? reinterpret_cast<uint32_t*>(sums + n_segments) : nullptr;
-  if (sums) {
+  const bool count = sums && n_rows * vocab * esz <= psa::kCountBytes;
+  uint32_t* n_left = count ? reinterpret_cast<uint32_t*>(sums + n_segments) : nullptr;
+  if (sums && !count) {
+    if (n_segments > 0 && cudaMemsetAsync(sums, 0, sizeof(double) * size_t(n_segments), st) != cudaSuccess)
+      return PSA_ERR_CUDA;
+  } else if (sums) {
     psa::dpo_logp_start_kernel<<<1, 1024, 0, st>>>(segment_ids, n_rows, fork_rows, n_forks, n_segments, out, sums, n_left);
   } else if (n_segments > 0 && cudaMemsetAsync(out, 0, sizeof(float) * size_t(n_segments), st) != cudaSuccess) {
     return PSA_ERR_CUDA;
@@ -257,6 +270,8 @@ psa_status_t run_logp(const void* logits, int32_t logits_dtype, int64_t n_rows, 
     psa::dpo_logp_kernel<__nv_bfloat16, 4><<<grid, psa::kLogpThreads, 0, st>>>(
         static_cast<const __nv_bfloat16*>(logits), vocab, row_stride, targets, segment_ids, fork_rows, fork_targets,
         fork_segments, n_forks, n_segments, out, sums, n_left, device_status);
+  if (sums && !count && n_segments > 0)
+    psa::dpo_logp_round_kernel<<<unsigned(n_segments + 127) / 128, 128, 0, st>>>(sums, out, n_segments);
   return psa::check_last_cuda_error("dpo_logp launch");
 }
 }  // namespace

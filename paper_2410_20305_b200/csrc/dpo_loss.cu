@@ -369,11 +369,10 @@ psa_status_t launch_logp_bwd(const T* logits, int64_t n_rows, int64_t vocab, int
                              const int32_t* fork_segments, int32_t n_forks, int32_t n_segments, const float* coef,
                              T* dlogits, int32_t* status, cudaStream_t stream) {
   auto kernel = dpo_logp_bwd_kernel<T, kThreads, kStaged, kPerSm>;
-  // (one CTA per SM: more than half of the SM's shared memory keeps a second one out)
-  constexpr size_t kAlone = 120 * 1024;
-  const size_t smem = kStaged ? size_t(vocab / Elem<T>::kVec) * 16 : (kPerSm == 1 ? kAlone : 0);
-  if (smem > 40 * 1024 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               int(kPerSm == 1 ? kAlone : size_t(kStagedMost))) != cudaSuccess)
+  // (One CTA per SM at kPerSm = 1 is the registers' doing: 1024 threads of more than 32.)
+  const size_t smem = kStaged ? size_t(vocab / Elem<T>::kVec) * 16 : 0;
+  if (smem > 40 * 1024 &&
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kStagedMost)) != cudaSuccess)
     return PSA_ERR_CUDA;
   kernel<<<unsigned(n_rows), kThreads, smem, stream>>>(logits, vocab, row_stride, targets, segment_ids, fork_rows,
                                                       fork_targets, fork_segments, n_forks, n_segments, coef, dlogits,

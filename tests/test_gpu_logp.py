@@ -127,7 +127,8 @@ def test_rows_that_begin_with_a_block_of_minus_infinity(dtype):
     assert np.abs(grad - ref).max() <= (2e-6 if dtype == torch.float32 else 2.0 ** -8)
 
 
-@pytest.mark.parametrize("dtype,vocab,rows", [(torch.float32, 3, 4000), (torch.bfloat16, 515, 3000), (torch.bfloat16, 4096 + 8, 1500)])
+@pytest.mark.parametrize("dtype,vocab,rows", [(torch.float32, 3, 4000), (torch.bfloat16, 515, 3000), (torch.bfloat16, 4096 + 8, 1500),
+                                              (torch.float32, 32768, 1024), (torch.float32, 32768, 1025)])   # 128 MB: the sums are rounded elsewhere
 def test_long_responses_are_summed_without_the_rounding_of_a_running_sum(dtype, vocab, rows):
     x, _ = wl.logits_and_tokens(rows, (vocab + 7) // 8 * 8, 31, 3.0 ** 0.5, dtype)
     rng = np.random.default_rng(4)
