@@ -18,9 +18,6 @@
 namespace psa {
 namespace {
 
-// 128 threads x 4 loads in flight measured best on B200 (6.86 TB/s on 8192 x 128256 bf16; 256 x 4: 6.71,
-// 512 x 4: 5.5, 1024 x 4: 4.6): small CTAs keep many rows in flight per SM and retire unevenly.
-constexpr int kLogpThreads = 128;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
@@ -113,7 +110,7 @@ __global__ void dpo_logp_round_kernel(const double* __restrict__ sums, float* __
 // fp32 107 -> 111) and the count of the live rows 4 us more; the extra launch costs 2 us, and the host as much.
 constexpr int64_t kCountBytes = int64_t(128) << 20;
 
-template <typename T, int kUnroll>
+template <typename T, int kUnroll, int kLogpThreads>
 __global__ void __launch_bounds__(kLogpThreads)
 dpo_logp_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_stride, const int32_t* __restrict__ targets,
                 const int32_t* __restrict__ segment_ids, const int32_t* __restrict__ fork_rows,
@@ -260,16 +257,27 @@ psa_status_t run_logp(const void* logits, int32_t logits_dtype, int64_t n_rows, 
     return PSA_ERR_CUDA;
   }
   if (n_rows == 0) return PSA_OK;
-  const unsigned grid = unsigned(n_rows);
   psa::ProfileScope prof(2, stream);
-  if (logits_dtype == PSA_DTYPE_F32)
-    psa::dpo_logp_kernel<float, 4><<<grid, psa::kLogpThreads, 0, st>>>(
-        static_cast<const float*>(logits), vocab, row_stride, targets, segment_ids, fork_rows, fork_targets,
-        fork_segments, n_forks, n_segments, out, sums, n_left, device_status);
-  else
-    psa::dpo_logp_kernel<__nv_bfloat16, 4><<<grid, psa::kLogpThreads, 0, st>>>(
-        static_cast<const __nv_bfloat16*>(logits), vocab, row_stride, targets, segment_ids, fork_rows, fork_targets,
-        fork_segments, n_forks, n_segments, out, sums, n_left, device_status);
+  auto run = [&](auto kernel, auto* x, int threads) {
+    kernel<<<unsigned(n_rows), threads, 0, st>>>(x, vocab, row_stride, targets, segment_ids, fork_rows, fork_targets,
+                                                 fork_segments, n_forks, n_segments, out, sums, n_left, device_status);
+  };
+  // Threads x loads in flight per thread.  Small CTAs keep many rows in flight per SM and retire unevenly, which suits
+  // many rows: 16215 x 128256 bf16, 2/3 live, 400 us with 128 x 4, 408 with 256 x 4, 484 with 512 x 4.  A few long rows
+  // are less than two waves of 1480 such CTAs, and a wave lasts as long as a row: 1800 x 128256 bf16 66 -> 60 us with
+  // 256 x 4.  fp32 rows have half the exponentials per byte and take more loads in flight from 64 KB on: 4096 x 50257
+  // 107 -> 85 us with 256 x 8, 8192 x 50257 171 -> 157, 4000 x 16384 36 -> 33, 3312 x 115288 (360 live) 54 -> 37; below,
+  // 128 x 4 stays better (6000 x 8192 27 against 29).
+  const int64_t row_bytes = vocab * esz;
+  if (logits_dtype == PSA_DTYPE_F32) {
+    const float* x = static_cast<const float*>(logits);
+    if (row_bytes >= 64 * 1024) run(psa::dpo_logp_kernel<float, 8, 256>, x, 256);
+    else run(psa::dpo_logp_kernel<float, 4, 128>, x, 128);
+  } else {
+    const __nv_bfloat16* x = static_cast<const __nv_bfloat16*>(logits);
+    if (row_bytes >= 128 * 1024 && n_rows <= 4096) run(psa::dpo_logp_kernel<__nv_bfloat16, 4, 256>, x, 256);
+    else run(psa::dpo_logp_kernel<__nv_bfloat16, 4, 128>, x, 128);
+  }
   if (sums && !count && n_segments > 0)
     psa::dpo_logp_round_kernel<<<unsigned(n_segments + 127) / 128, 128, 0, st>>>(sums, out, n_segments);
   return psa::check_last_cuda_error("dpo_logp launch");

@@ -128,7 +128,8 @@ def test_rows_that_begin_with_a_block_of_minus_infinity(dtype):
 
 
 @pytest.mark.parametrize("dtype,vocab,rows", [(torch.float32, 3, 4000), (torch.bfloat16, 515, 3000), (torch.bfloat16, 4096 + 8, 1500),
-                                              (torch.float32, 32768, 1024), (torch.float32, 32768, 1025)])   # 128 MB: the sums are rounded elsewhere
+                                              (torch.float32, 32768, 1024), (torch.float32, 32768, 1025), (torch.float32, 16383, 300),
+                                              (torch.bfloat16, 65535, 500), (torch.bfloat16, 65544, 500)])   # 128 MB: the sums are rounded elsewhere
 def test_long_responses_are_summed_without_the_rounding_of_a_running_sum(dtype, vocab, rows):
     x, _ = wl.logits_and_tokens(rows, (vocab + 7) // 8 * 8, 31, 3.0 ** 0.5, dtype)
     rng = np.random.default_rng(4)
