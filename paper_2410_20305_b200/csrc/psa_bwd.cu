@@ -362,9 +362,14 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       if (e & 1) {
         const int lo = kv_local - q0 - c0;                   // first allowed column (causal), relative to c0
         const int hi = qend - q0 - c0;                       // one past the last allowed column
-        const uint32_t span = hi > lo ? uint32_t(hi - lo) : 0u;
+        // one bit per column: a bit costs one instruction to test, the interval two
+        auto below = [](int n) { return n >= 32 ? 0xffffffffu : (n <= 0 ? 0u : (1u << n) - 1u); };   // bits [0, n)
 #pragma unroll
-        for (int i = 0; i < 64; ++i) p[i] = (uint32_t(i - lo) < span) ? p[i] : 0.f;
+        for (int j = 0; j < 2; ++j) {
+          const uint32_t allowed = below(hi - 32 * j) & ~below(lo - 32 * j);
+#pragma unroll
+          for (int i = 0; i < 32; ++i) p[32 * j + i] = (allowed >> i & 1u) ? p[32 * j + i] : 0.f;
+        }
       }
       {
         // bf16 pairs: this half's 64 probabilities go to the first 32 of the 64 S^T columns this

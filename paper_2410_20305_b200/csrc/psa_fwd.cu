@@ -286,24 +286,23 @@ psa_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       const bool precise = (e & 2) != 0;
       mbar_wait(bar(BAR_S_FULL), g & 1, wctx);
       tc_fence_after();
-      // Allowed keys of this row in a PARTIAL tile, relative to the tile: [0, a) and [b, b + span).
-      int a = kTile, b = 0;
-      uint32_t span = 0;
+      // Allowed keys of this row in a PARTIAL tile, relative to the tile: [0, a) and [b, end), as one bit per
+      // column of the thread's two 32-column chunks (a bit costs one instruction to test, the two intervals four).
+      // Warp-uniform class of each chunk: 0 = every lane allows every column (no masking), 1 = mixed (mask per
+      // element), 2 = no lane allows any column (skipped: no load, no exponential).  On a causal diagonal tile this
+      // skips 3/8 of the exponentials.
+      uint32_t cls = 0, allowed[2] = {0xffffffffu, 0xffffffffu};
       if (e & 1) {
+        int a, b = 0, end = 0;
         if (q_local < rec.rs) { a = q_local + 1 - k0; }
-        else { a = rec.cs - k0; b = rec.rs - k0; span = uint32_t(q_local + 1 - rec.rs); }
-      }
-      // Warp-uniform class of this warp's two 32-column chunks: 0 = every lane allows every column
-      // (no masking), 1 = mixed (mask per element), 2 = no lane allows any column (skipped: no load,
-      // no exponential).  On a causal diagonal tile this skips 3/8 of the exponentials.
-      uint32_t cls = 0;
-      if (e & 1) {
+        else { a = rec.cs - k0; b = rec.rs - k0; end = q_local + 1 - k0; }
+        auto below = [](int n) { return n >= 32 ? 0xffffffffu : (n <= 0 ? 0u : (1u << n) - 1u); };   // bits [0, n)
 #pragma unroll
         for (int sub = 0; sub < 2; ++sub) {
-          const int lo = hfz * 64 + sub * 32, hi = lo + 32;
-          const bool all_ok = (hi <= a) || (lo >= b && uint32_t(hi - b) <= span);
-          const bool none_ok = (lo >= a) && (span == 0u || hi <= b || (lo >= b && uint32_t(lo - b) >= span));
-          const uint32_t cc = __all_sync(0xffffffffu, all_ok) ? 0u : (__all_sync(0xffffffffu, none_ok) ? 2u : 1u);
+          const int lo = hfz * 64 + sub * 32;
+          allowed[sub] = below(a - lo) | (below(end - lo) & ~below(b - lo));
+          const uint32_t cc = __all_sync(0xffffffffu, allowed[sub] == 0xffffffffu)
+                                  ? 0u : (__all_sync(0xffffffffu, allowed[sub] == 0u) ? 2u : 1u);
           cls |= cc << (2 * sub);
         }
       }
@@ -315,11 +314,7 @@ psa_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         tmem_ld32_wait(tmem + lane_base + col_s + sub * 32, v);
         if (chunk_class(sub) == 1u) {
 #pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            const int col = hfz * 64 + sub * 32 + i;
-            const bool ok = (col < a) || (uint32_t(col - b) < span);
-            x[i] = ok ? __uint_as_float(v[i]) : -INFINITY;
-          }
+          for (int i = 0; i < 32; ++i) x[i] = (allowed[sub] >> i & 1u) ? __uint_as_float(v[i]) : -INFINITY;
         } else {   // class 0; callers never use the values of a class-2 chunk
 #pragma unroll
           for (int i = 0; i < 32; ++i) x[i] = __uint_as_float(v[i]);
@@ -407,11 +402,8 @@ psa_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           float x[16];
           if (cc == 1u) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const int col = hfz * 64 + ch * 16 + i;
-              const bool ok = (col < a) || (uint32_t(col - b) < span);
-              x[i] = ok ? __uint_as_float(v[i]) : -INFINITY;
-            }
+            for (int i = 0; i < 16; ++i)
+              x[i] = (allowed[ch >> 1] >> ((ch & 1) * 16 + i) & 1u) ? __uint_as_float(v[i]) : -INFINITY;
           } else {
 #pragma unroll
             for (int i = 0; i < 16; ++i) x[i] = __uint_as_float(v[i]);
