@@ -717,7 +717,7 @@ def main():
                      "algorithmic_flops": flops_bwd, "algorithmic_bytes": T * (4 * Hq + 4 * Hkv) * d * 2,
                      "traffic": traffic, "traffic_source": traffic_note},
         "clocks": clk,
-        "gpu_launches": n_pass * (4 if args.no_logp else 5),
+        "gpu_launches": n_pass * (4 if args.no_logp else 6),
         "paired_layout": paired,
         "workloads": others,
         "dpo_logp_all_rows": all_rows,

@@ -131,8 +131,8 @@ void order_backward(psa_plan_t* p, const std::vector<std::vector<int32_t>>& tile
   //   16700 tokens, 8/2 heads of 128 (262)          1383 / 1262 / 1374 / 1482 in short runs, 1376 / 1389 in long ones,
   //   where the power limit sets the clock: a prediction of less than 10 % is not worth it.
   //   5061 tokens, 32/8 heads of 128 (328)          264 / 270 / 354 / 575
-  if (part != &p->whole) {   // (a part runs under the copies of another: no simulation, only what fits at once)
-    while (part->bwd_split < 4 && ctas.size() * part->bwd_split * 2 <= size_t(n_sm) * 33 / 37) part->bwd_split *= 2;
+  if (part != &p->whole) {
+    part->bwd_split = p->whole.bwd_split;   // dk and dv are summed in the same order, and come out the same, as for the whole
   } else if (ctas.size() <= 2 * size_t(n_sm)) {
     const int64_t iter_ns = p->d == 128 ? 2050 : 1600, fixed_ns = p->d == 128 ? 8000 : 7000, combine_ns = 3000;
     const int64_t group = p->Hq / p->Hkv;
