@@ -121,6 +121,20 @@ def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
+def _temporary(n, dtype, device, stream):
+    """A device buffer that the library uses on `stream` and that the caller drops on return.  torch gives a freed
+    block to the next tensor of the stream that the block was allocated on, so it is allocated on the stream of the
+    call: whoever owns it before or after has its work ordered against the call's.  (A graph captured by other means
+    than torch's has no pool that keeps such a block: there the caller passes the buffer.)"""
+    import torch
+    if stream is None or int(stream) == _stream(None):
+        return torch.empty(n, dtype=dtype, device=device)
+    # handles 0 and 1 both name the default stream
+    own = torch.cuda.default_stream(device) if int(stream) in (0, 1) else torch.cuda.ExternalStream(int(stream), device=device)
+    with torch.cuda.stream(own):
+        return torch.empty(n, dtype=dtype, device=device)
+
+
 def _want(t, name, shape, dtype, cuda=True, placement=True):
     """Raises ValueError unless tensor `t` has exactly this shape and dtype, is contiguous and
     lives where the call needs it.  The kernels size their tensor maps and grids from the plan
@@ -291,9 +305,11 @@ def psa_selftest_bounds(status, result, stream=None):
 
 
 def dpo_logp(logits, targets, segment_ids, n_segments, fork_rows=None, fork_targets=None, fork_segments=None,
-             out=None, status=None, stream=None):
+             out=None, status=None, stream=None, scratch=None):
     """logits [n_rows, vocab] fp32 or bf16 (rows may be strided), targets / segment_ids
-    int32 [n_rows], optional fork arrays int32 [n_forks] -> out fp32 [n_segments]."""
+    int32 [n_rows], optional fork arrays int32 [n_forks] -> out fp32 [n_segments].
+    `scratch` (optional): a CUDA buffer of at least 8 * (n_segments + 1) bytes for the fp64 sums,
+    in use until the call's work on the stream has ended."""
     import torch
     assert logits.is_cuda and logits.dim() == 2 and logits.stride(1) == 1
     dt = {torch.float32: PSA_DTYPE_F32, torch.bfloat16: PSA_DTYPE_BF16}[logits.dtype]
@@ -308,7 +324,10 @@ def dpo_logp(logits, targets, segment_ids, n_segments, fork_rows=None, fork_targ
         fork_rows = fork_targets = fork_segments = None
     if out is None:
         out = torch.empty(n_segments, dtype=torch.float32, device=logits.device)
-    scratch = torch.empty(n_segments + 1, dtype=torch.float64, device=logits.device)
+    if scratch is None:
+        scratch = _temporary(n_segments + 1, torch.float64, logits.device, stream)
+    if not scratch.is_cuda or scratch.numel() * scratch.element_size() < 8 * (n_segments + 1):
+        raise ValueError("scratch: a CUDA buffer of at least %d bytes is needed" % (8 * (n_segments + 1)))
     _check("dpo_logp", load_library().dpo_logp_f64sum(
         _ptr(logits), dt, n_rows, vocab, logits.stride(0) if n_rows > 1 else vocab, _ptr(targets), _ptr(segment_ids),
         _ptr(fork_rows), _ptr(fork_targets), _ptr(fork_segments), n_forks, n_segments, _ptr(out), _ptr(scratch),

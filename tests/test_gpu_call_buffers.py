@@ -1,0 +1,91 @@
+"""Buffers that the binding allocates for one call: they belong to the stream that the call runs on, so neither
+another stream's tensors nor a call on another stream get them while the call's kernels still use them."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import psa_oracle as orc
+from paper_2410_20305_b200 import binding as B
+from paper_2410_20305_b200 import workloads as wl
+
+from gpu_util import read_status
+
+pytestmark = pytest.mark.gpu
+
+
+class _Recorder:
+    """The library, with the arguments of one entry point's calls written down."""
+
+    def __init__(self, name):
+        self._lib, self._name, self.calls = B.load_library(), name, []
+
+    def __getattr__(self, name):
+        fn = getattr(self._lib, name)
+        if name != self._name:
+            return fn
+        return lambda *a: (self.calls.append(a), fn(*a))[1]
+
+
+def _blocks_of(bytes_, n=16):
+    """Addresses that the current stream's next tensors of this size get."""
+    return [t.data_ptr() for t in [torch.empty(bytes_, dtype=torch.uint8, device="cuda") for _ in range(n)]]
+
+
+def _device(a):
+    return torch.as_tensor(np.asarray(a, dtype=np.int32)).cuda()
+
+
+def _logp_inputs(rows, vocab, n_segments, seed):
+    x, _ = wl.logits_and_tokens(rows, vocab, seed, 3.0 ** 0.5, torch.bfloat16)
+    rng = np.random.default_rng(seed)
+    targets = rng.integers(0, vocab, rows).astype(np.int32)
+    seg = np.where(np.arange(rows) % 5 == 0, -1, rng.integers(0, n_segments, rows)).astype(np.int32)
+    return (x.cuda(), _device(targets), _device(seg), n_segments), orc.dpo_logp(wl.to_f64(x), targets, seg, n_segments, [], [], [])
+
+
+def test_dpo_logp_on_a_stream_that_is_not_current(monkeypatch):
+    args, want = _logp_inputs(300, 1024, 6, 1)
+    rec = _Recorder("dpo_logp_f64sum")
+    monkeypatch.setattr(B, "load_library", lambda: rec)
+    side = torch.cuda.Stream()
+    a = torch.randn((4096, 4096), device="cuda", dtype=torch.bfloat16)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        for _ in range(40):
+            a @ a                                      # the side stream is busy while the call returns
+    out = torch.zeros(6, device="cuda")
+    torch.cuda.current_stream().synchronize()
+    B.dpo_logp(*args, out=out, stream=side.cuda_stream)
+    assert rec.calls[-1][13] not in _blocks_of(8 * 7)
+    side.synchronize()
+    assert np.abs(out.cpu().double().numpy() - want).max() <= 1e-4 * np.abs(want).max()
+
+
+def test_dpo_logp_on_two_streams_at_once():
+    # policy and reference logits; many calls, so that they overlap
+    sets = [_logp_inputs(700, 2048, 6, seed) for seed in (2, 3)]
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    torch.cuda.synchronize()
+    outs = [[torch.zeros(6, device="cuda") for _ in range(50)] for _ in sets]
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    for i in range(50):
+        for (args, _), stream, out in zip(sets, streams, outs):
+            B.dpo_logp(*args, out=out[i], status=status, stream=stream.cuda_stream)
+    assert read_status(status) == 0
+    for (_, want), out in zip(sets, outs):
+        got = torch.stack(out).cpu().double().numpy()
+        assert np.abs(got - want).max() <= 1e-4 * np.abs(want).max()
+
+
+def test_dpo_logp_scratch_of_the_caller(monkeypatch):
+    args, want = _logp_inputs(300, 1024, 6, 4)
+    rec = _Recorder("dpo_logp_f64sum")
+    monkeypatch.setattr(B, "load_library", lambda: rec)
+    scratch = torch.full((7,), float("nan"), dtype=torch.float64, device="cuda")   # contents on entry do not matter
+    got = B.dpo_logp(*args, scratch=scratch).cpu().double().numpy()
+    assert rec.calls[-1][13] == scratch.data_ptr()
+    assert np.abs(got - want).max() <= 1e-4 * np.abs(want).max()
+    for small in (scratch[:6], torch.zeros(7, dtype=torch.float64)):
+        with pytest.raises(ValueError):
+            B.dpo_logp(*args, scratch=small)
