@@ -135,6 +135,7 @@ dpo_logp_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_stride,
       __threadfence();
     }
     if (__shfl_sync(0xffffffffu, before, 0) != 1u) return;
+    __syncwarp();   // lane 0 has fenced for the other lanes: only this orders their reads behind it (a shuffle does not)
     for (int g = threadIdx.x & 31; g < n_segments; g += 32) out[g] = float(__ldcg(sums + g));
   };
   if (seg < 0 && !forked) return;      // dead row: its logits are never read

@@ -143,3 +143,19 @@ def test_long_responses_are_summed_without_the_rounding_of_a_running_sum(dtype, 
     # per row half an ulp of its fp32 log-sum-exp (below 16: 5e-7) and the exponentials' error of the same size, with
     # signs that differ from row to row; then one rounding of the sum (6e-8 of it)
     assert got[3] == 0 and (np.abs(got - want) <= 1e-6 * 4 * np.sqrt(rows) + 6e-8 * np.abs(want)).all()
+
+
+@pytest.mark.parametrize("n_segments", [1, 31, 33, 70, 1000])
+def test_the_last_row_rounds_every_sum(n_segments):
+    # small launches: the row that finishes last rounds all sums, a lane for each; every sum has to hold every row's term
+    rows, vocab = 900, 512
+    x, _ = wl.logits_and_tokens(rows, vocab, 5, 3.0 ** 0.5, torch.bfloat16)
+    rng = np.random.default_rng(n_segments)
+    targets = rng.integers(0, vocab, rows).astype(np.int32)
+    seg = rng.integers(-1, n_segments, rows).astype(np.int32)
+    args = x.cuda(), _dev(targets), _dev(seg), n_segments
+    want = orc.dpo_logp(wl.to_f64(x), targets, seg, n_segments)
+    for got in [B.dpo_logp(*args, out=torch.full((n_segments,), 7.0, device="cuda")) for _ in range(30)]:
+        got = got.cpu().double().numpy()
+        # up to 900 terms, each off by an ulp of its fp32 log-sum-exp (1e-6); the rounding of a sum of at most 900 x 15
+        assert (np.abs(got - want) <= 1e-6 * 4 * np.sqrt(rows) + 6e-8 * np.abs(want)).all()
