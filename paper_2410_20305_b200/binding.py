@@ -326,7 +326,7 @@ def dpo_logp(logits, targets, segment_ids, n_segments, fork_rows=None, fork_targ
         out = torch.empty(n_segments, dtype=torch.float32, device=logits.device)
     if scratch is None:
         scratch = _temporary(n_segments + 1, torch.float64, logits.device, stream)
-    if not scratch.is_cuda or scratch.numel() * scratch.element_size() < 8 * (n_segments + 1):
+    elif not scratch.is_cuda or scratch.numel() * scratch.element_size() < 8 * (n_segments + 1):
         raise ValueError("scratch: a CUDA buffer of at least %d bytes is needed" % (8 * (n_segments + 1)))
     _check("dpo_logp", load_library().dpo_logp_f64sum(
         _ptr(logits), dt, n_rows, vocab, logits.stride(0) if n_rows > 1 else vocab, _ptr(targets), _ptr(segment_ids),

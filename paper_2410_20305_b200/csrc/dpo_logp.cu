@@ -4,8 +4,10 @@
 // (max, sum of exp) per thread in fp32, merges across the warp with shuffles and
 // across warps through shared memory, and adds  logit[target] - lse  into
 // out[segment] with one atomic per scored label, or, where the caller gives scratch for them, into
-// fp64 sums that are rounded into out at the end: a response of 250 tokens is then off by its
-// lse's and one final rounding (3e-8) instead of 250 (1e-7 to 4e-7).
+// fp64 sums: a response of 250 tokens is then off by its lse's and one final rounding (3e-8) instead
+// of 250 (1e-7 to 4e-7).  Every term is at most 0, so a sum only falls while its rows arrive, and
+// so does its rounding to fp32: out[segment] is the lowest of the roundings that the rows have seen,
+// whatever their order, and nothing has to wait for the last row.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -19,7 +21,7 @@ namespace psa {
 namespace {
 
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kLn2 = 0.6931471805599453f;
+constexpr double kLn2 = 0.6931471805599453;
 
 __device__ __forceinline__ float ex2_approx(float x) {
   float y;
@@ -66,49 +68,36 @@ struct MaxSum {
   float m, s;
   __device__ void merge(float m2, float s2) {
     const float mn = fmaxf(m, m2);
-    if (mn == -INFINITY) return;
+    if (mn == -INFINITY) {   // nothing finite on either side: both sums are 0, or NaN where a logit was
+      s += s2;
+      return;
+    }
     s = s * ex2_approx(m - mn) + s2 * ex2_approx(m2 - mn);
     m = mn;
   }
 };
 
-// Clears out and the fp64 sums and counts the rows that score anything; one block.
-__global__ void __launch_bounds__(1024)
-dpo_logp_start_kernel(const int32_t* __restrict__ segment_ids, int64_t n_rows, const int32_t* __restrict__ fork_rows,
-                      int32_t n_forks, int32_t n_segments, float* __restrict__ out, double* __restrict__ sums,
-                      uint32_t* __restrict__ n_left) {
-  __shared__ uint32_t s_live;
-  if (threadIdx.x == 0) s_live = 0;
-  for (int g = threadIdx.x; g < n_segments; g += 1024) {
+// One launch for both arrays.  With add_f64 it replaced a pass over the segment ids that counted the live rows, the count
+// of every row at its end and a last row that rounded all sums (small launches), or a second kernel that did (large ones);
+// us of the whole call, before -> now, and with fp32 atomics behind a memset: 6335 x 6215 bf16 24.0 -> 15.3 (18.4),
+// 12000 x 1000 bf16 with 100 responses 21.9 -> 13.6 (16.0), with 4000 responses 47.2 -> 10.5 (10.4), 700 x 1024 fp32
+// 6.9 -> 4.7 (6.3), 8192 x 50257 fp32 147.5 -> 143.3 (167).
+__global__ void dpo_logp_clear_kernel(float* __restrict__ out, double* __restrict__ sums, int32_t n_segments) {
+  const int32_t g = blockIdx.x * blockDim.x + threadIdx.x;
+  if (g < n_segments) {
     out[g] = 0.f;
     sums[g] = 0.0;
   }
-  __syncthreads();
-  uint32_t live = 0;
-#pragma unroll 8
-  for (int64_t t = threadIdx.x; t < n_rows; t += 1024) live += segment_ids[t] >= 0;
-  for (int f = threadIdx.x; f < n_forks; f += 1024) {   // a row that only forks score, once
-    const int64_t row = fork_rows[f];
-    if (row < 0 || row >= n_rows || segment_ids[row] >= 0) continue;
-    bool first = true;
-    for (int e = 0; e < f && first; ++e) first = fork_rows[e] != row;
-    live += first;
-  }
-  live = __reduce_add_sync(0xffffffffu, live);
-  if ((threadIdx.x & 31) == 0) atomicAdd(&s_live, live);
-  __syncthreads();
-  if (threadIdx.x == 0) *n_left = s_live;
 }
 
-__global__ void dpo_logp_round_kernel(const double* __restrict__ sums, float* __restrict__ out, int32_t n_segments) {
-  const int32_t g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g < n_segments) out[g] = float(sums[g]);
+// Adds a term (a log-probability) to the fp64 sum and lowers out to its rounding.
+__device__ __forceinline__ void add_f64(double* sum, float* out, double term) {
+  // a probability that rounding has put above 1 counts as 1, so that the sum never rises (a NaN stays one)
+  if (term > 0.0) term = 0.0;
+  const double now = atomicAdd(sum, term) + term;
+  // The bits of floats that are not positive grow as the values fall; the largest of all is a NaN.
+  atomicMax(reinterpret_cast<uint32_t*>(out), now == now ? __float_as_uint(float(now)) : 0xffffffffu);
 }
-
-// Logits up to this size let the last live row round the fp64 sums; above, a kernel of its own does.  The wait of
-// every row's CTA for its place in the count costs 3.5 % of the kernel (16215 x 128256 bf16 265 -> 274 us, 4096 x 50257
-// fp32 107 -> 111) and the count of the live rows 4 us more; the extra launch costs 2 us, and the host as much.
-constexpr int64_t kCountBytes = int64_t(128) << 20;
 
 template <typename T, int kUnroll, int kLogpThreads>
 __global__ void __launch_bounds__(kLogpThreads)
@@ -116,7 +105,7 @@ dpo_logp_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_stride,
                 const int32_t* __restrict__ segment_ids, const int32_t* __restrict__ fork_rows,
                 const int32_t* __restrict__ fork_targets, const int32_t* __restrict__ fork_segments, int32_t n_forks,
                 int32_t n_segments, float* __restrict__ out, double* __restrict__ sums /* [n_segments], or null */,
-                uint32_t* __restrict__ n_left /* live rows not finished, or null */, int32_t* __restrict__ status) {
+                int32_t* __restrict__ status) {
   constexpr int E = Vec<T>::kElems;
   const int64_t row = blockIdx.x;
   const int32_t seg = segment_ids[row];
@@ -124,20 +113,6 @@ dpo_logp_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_stride,
   bool forked = false;
   for (int f = threadIdx.x & 31; f < n_forks; f += 32) forked |= fork_rows[f] == row;
   forked = __any_sync(0xffffffffu, forked);
-  // In a small launch with fp64 sums every live row counts itself when it has added its own; the last one rounds them
-  // all.
-  auto finish = [&]() {   // by one warp
-    if (!n_left) return;
-    uint32_t before = 0;
-    if ((threadIdx.x & 31) == 0) {
-      __threadfence();
-      before = atomicSub(n_left, 1u);
-      __threadfence();
-    }
-    if (__shfl_sync(0xffffffffu, before, 0) != 1u) return;
-    __syncwarp();   // lane 0 has fenced for the other lanes: only this orders their reads behind it (a shuffle does not)
-    for (int g = threadIdx.x & 31; g < n_segments; g += 32) out[g] = float(__ldcg(sums + g));
-  };
   if (seg < 0 && !forked) return;      // dead row: its logits are never read
 
   const T* x = logits + row * row_stride;
@@ -184,8 +159,10 @@ dpo_logp_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_stride,
     acc.m = mn;
     acc.s = s;
   }
-  for (int64_t j = n_vec * E + threadIdx.x; j < vocab; j += kLogpThreads)  // ragged tail of the row
-    acc.merge(Vec<T>::load1(x + j) * kLog2e, 1.f);
+  for (int64_t j = n_vec * E + threadIdx.x; j < vocab; j += kLogpThreads) {  // ragged tail of the row
+    const float y = Vec<T>::load1(x + j), m2 = y * kLog2e;
+    if (y != -INFINITY) acc.merge(m2, ex2_approx(fmaf(y, kLog2e, -m2)));     // (what the product's rounding has left)
+  }
 
   // Warp merge by shuffles, then across warps through shared memory.
 #pragma unroll
@@ -208,13 +185,16 @@ dpo_logp_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_stride,
       t.merge(m2, s2);
     }
     if (lane == 0) {
-      const float lse = (t.m + log2f(t.s)) * kLn2;  // natural log of sum exp(x)
+      // log2 of the probability, the maximum taken off before anything is rounded to fp32: the term of a token
+      // that takes nearly all of the probability is then near 0 itself, not the difference of two numbers like 50
+      const double m = t.m, log2s = log2f(t.s);
       auto score = [&](int32_t y, int32_t g) {
         if (g < 0) return;
         if (g >= n_segments) { if (status) atomicOr(status, PSA_DEVSTAT_BAD_SEGMENT); return; }
         if (y < 0 || y >= vocab) { if (status) atomicOr(status, PSA_DEVSTAT_BAD_TARGET); return; }
-        if (sums) atomicAdd(sums + g, double(Vec<T>::load1(x + y)) - double(lse));
-        else atomicAdd(out + g, Vec<T>::load1(x + y) - lse);
+        const double term = (fma(double(Vec<T>::load1(x + y)), double(kLog2e), -m) - log2s) * kLn2;
+        if (sums) add_f64(sums + g, out + g, term);
+        else atomicAdd(out + g, float(term));
       };
       score(targets[row], seg);
       if (forked) {
@@ -223,8 +203,6 @@ dpo_logp_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_stride,
           if (fork_rows[f] == row) score(fork_targets[f], fork_segments[f]);
       }
     }
-    __syncwarp();
-    finish();
   }
 }
 
@@ -247,21 +225,15 @@ psa_status_t run_logp(const void* logits, int32_t logits_dtype, int64_t n_rows, 
   if ((reinterpret_cast<uintptr_t>(logits) & 15) || (n_rows > 1 && ((row_stride * esz) & 15))) return PSA_ERR_ALIGNMENT;
   cudaStream_t st = cudaStream_t(stream);
   if (n_rows == 0) sums = nullptr;   // nothing runs that would round them
-  const bool count = sums && n_rows * vocab * esz <= psa::kCountBytes;
-  uint32_t* n_left = count ? reinterpret_cast<uint32_t*>(sums + n_segments) : nullptr;
-  if (sums && !count) {
-    if (n_segments > 0 && cudaMemsetAsync(sums, 0, sizeof(double) * size_t(n_segments), st) != cudaSuccess)
-      return PSA_ERR_CUDA;
-  } else if (sums) {
-    psa::dpo_logp_start_kernel<<<1, 1024, 0, st>>>(segment_ids, n_rows, fork_rows, n_forks, n_segments, out, sums, n_left);
-  } else if (n_segments > 0 && cudaMemsetAsync(out, 0, sizeof(float) * size_t(n_segments), st) != cudaSuccess) {
+  if (sums && n_segments > 0)
+    psa::dpo_logp_clear_kernel<<<unsigned(n_segments + 127) / 128, 128, 0, st>>>(out, sums, n_segments);
+  else if (n_segments > 0 && cudaMemsetAsync(out, 0, sizeof(float) * size_t(n_segments), st) != cudaSuccess)
     return PSA_ERR_CUDA;
-  }
   if (n_rows == 0) return PSA_OK;
   psa::ProfileScope prof(2, stream);
   auto run = [&](auto kernel, auto* x, int threads) {
     kernel<<<unsigned(n_rows), threads, 0, st>>>(x, vocab, row_stride, targets, segment_ids, fork_rows, fork_targets,
-                                                 fork_segments, n_forks, n_segments, out, sums, n_left, device_status);
+                                                 fork_segments, n_forks, n_segments, out, sums, device_status);
   };
   // Threads x loads in flight per thread.  Small CTAs keep many rows in flight per SM and retire unevenly, which suits
   // many rows: 16215 x 128256 bf16, 2/3 live, 400 us with 128 x 4, 408 with 256 x 4, 484 with 512 x 4.  A few long rows
@@ -279,8 +251,6 @@ psa_status_t run_logp(const void* logits, int32_t logits_dtype, int64_t n_rows, 
     if (row_bytes >= 128 * 1024 && n_rows <= 4096) run(psa::dpo_logp_kernel<__nv_bfloat16, 4, 256>, x, 256);
     else run(psa::dpo_logp_kernel<__nv_bfloat16, 4, 128>, x, 128);
   }
-  if (sums && !count && n_segments > 0)
-    psa::dpo_logp_round_kernel<<<unsigned(n_segments + 127) / 128, 128, 0, st>>>(sums, out, n_segments);
   return psa::check_last_cuda_error("dpo_logp launch");
 }
 }  // namespace

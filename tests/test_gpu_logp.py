@@ -159,3 +159,28 @@ def test_the_last_row_rounds_every_sum(n_segments):
         got = got.cpu().double().numpy()
         # up to 900 terms, each off by an ulp of its fp32 log-sum-exp (1e-6); the rounding of a sum of at most 900 x 15
         assert (np.abs(got - want) <= 1e-6 * 4 * np.sqrt(rows) + 6e-8 * np.abs(want)).all()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("vocab", [1, 7, 1000, 16392])
+def test_terms_at_the_ends_of_their_range(dtype, vocab):
+    """Responses of tokens that take all of the probability (terms of 0, where rounding must not add up), of a token
+    that is impossible (-inf), and with a NaN among the logits; the others keep their values."""
+    rows, stride = 400, (vocab + 7) // 8 * 8
+    x, _ = wl.logits_and_tokens(rows, stride, 12, 3.0 ** 0.5, dtype)
+    targets = np.random.default_rng(1).integers(0, vocab, rows).astype(np.int32)
+    seg = (np.arange(rows) // 100).astype(np.int32)
+    at = torch.as_tensor(targets[:100]).long()
+    x[torch.arange(100), at] = 150 + 7.3 * x[torch.arange(100), at]      # response 0: all certain
+    x[150, targets[150]] = -float("inf")                                 # response 1 (vocab 1: no probability left at all)
+    x[250, vocab // 2] = float("nan")                                    # response 2
+    got = B.dpo_logp(x.cuda()[:, :vocab], _dev(targets), _dev(seg), 5).cpu().double().numpy()
+    with np.errstate(invalid="ignore", divide="ignore"):
+        want = orc.dpo_logp(wl.to_f64(x)[:, :vocab], targets, seg, 5)
+    # per certain row the exponential's error (2^-22), all of the same sign at worst
+    assert abs(got[0] - want[0]) <= 100 * 5e-7, (got[0], want[0])
+    assert np.isnan(got[1]) if vocab == 1 else got[1] == -np.inf
+    assert np.isnan(got[2])
+    # (vocab 1: log2 of a sum that should be 1, with the exponential's error)
+    assert abs(got[3] - want[3]) <= 1e-6 * 4 * 10 + 6e-8 * abs(want[3]), (got[3], want[3])
+    assert got[4] == 0 and (got[[0, 3]] <= 0).all()
