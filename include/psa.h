@@ -159,6 +159,13 @@ psa_status_t psa_plan_export(const psa_plan_t* plan, int32_t direction,
                              int32_t* tiles, int32_t* entries);
 
 /*
+ * psa_plan_launch -- how psa_fwd and psa_bwd divide the plan's work (tests, tools); any output may
+ * be NULL.  fwd_items_per_cta: (query tile, query head) items per CTA of the forward, 1 or 2;
+ * bwd_ctas_per_pair: CTAs that share one (key tile, kv head) pair of the backward, 1, 2, 4 or 8.
+ */
+psa_status_t psa_plan_launch(const psa_plan_t* plan, int32_t* fwd_items_per_cta, int32_t* bwd_ctas_per_pair);
+
+/*
  * psa_fwd -- attention forward under the plan's mask (Section 3.1).
  *   S = scale * Q K^T on the live tiles, softmax over the allowed keys of each
  *   row in fp32, O = P V;  lse[h][t] = log sum_j exp(S[t][j])  (natural log).

@@ -27,7 +27,7 @@ EXPORTED_SYMBOLS = (
     "psa_bwd_static_scratch", "dpo_loss", "dpo_logp_bwd", "psa_pack_ffd", "psa_position_ids", "psa_rope",
     "psa_step_host_arena_bytes", "psa_step_host", "simpo_loss", "orpo_loss", "psa_bwd_f32",
     "psa_check_device_status", "psa_selftest_wait_expiry", "psa_logp_labels", "psa_pack_ffd_emit",
-    "psa_selftest_bounds", "dpo_logp_f64sum",
+    "psa_selftest_bounds", "dpo_logp_f64sum", "psa_plan_launch",
 )
 
 
@@ -65,6 +65,7 @@ def load_library():
                                    C.POINTER(C.c_size_t)]
     lib.psa_plan_counts.argtypes = [vp, i32, C.POINTER(i32), C.POINTER(i32)]
     lib.psa_plan_export.argtypes = [vp, i32, vp, vp]
+    lib.psa_plan_launch.argtypes = [vp, C.POINTER(i32), C.POINTER(i32)]
     lib.psa_fwd.argtypes = [vp] * 8
     lib.psa_bwd.argtypes = [vp] * 13
     lib.psa_bwd_static_scratch.argtypes = [vp] * 12
@@ -201,6 +202,12 @@ class Plan:
         entries = np.zeros(max(ne.value, 1), dtype=np.int32)
         _check("psa_plan_export", lib.psa_plan_export(self._h, direction, tiles.ctypes.data, entries.ctypes.data))
         return tiles[:nt.value], entries[:ne.value]
+
+    def launch(self):
+        """(work items per CTA of the forward, CTAs per (key tile, kv head) pair of the backward)."""
+        items, ctas = C.c_int32(), C.c_int32()
+        _check("psa_plan_launch", load_library().psa_plan_launch(self._h, C.byref(items), C.byref(ctas)))
+        return items.value, ctas.value
 
     def close(self):
         if self._h:

@@ -36,7 +36,6 @@ using namespace dev;
 
 constexpr int kFwdThreads = 384;
 constexpr int kSoftmaxThreads = 256;
-constexpr int kOneItemMost = 1184;   // four items for each of the 296 CTAs that 148 SMs hold
 // Register split of the 80 per thread the launch bound allows: the first warpgroup (producer,
 // issuer) gives registers to the two softmax warpgroups.
 constexpr int kRegsWg0 = 32, kRegsSoftmax = 104;
@@ -682,11 +681,7 @@ psa_status_t launch_fwd_t(const psa_plan_t* plan, const PlanPart& part, const vo
   prm.Hkv = plan->Hkv;
   prm.n_items = part.n_q_tiles * plan->Hq;
   prm.scale_log2 = plan->scale * 1.4426950408889634f;
-  // Two items per CTA pay the CTA's fixed costs once for both; one per CTA spreads a short list over more of the 296
-  // CTAs that the chip holds.  us, two -> one: 10505 tokens, 4 heads of 64 (332 items) 130 -> 65; 2954 tokens, 32 heads
-  // of 128 (768) 63 -> 53; 7965 tokens, 16 heads of 64 (1040) 56.6 -> 52.9; 5061 tokens, 32 heads of 128 (1312)
-  // 96.6 -> 100.4; 7727 tokens (2176) 79.7 -> 88.0; 31041 tokens (7904) 965 -> 1019.
-  prm.items_per_cta = prm.n_items <= kOneItemMost ? 1 : 2;
+  prm.items_per_cta = part.fwd_items_per_cta;
   const unsigned grid = unsigned(prm.n_items + prm.items_per_cta - 1) / unsigned(prm.items_per_cta);
   {
     ProfileScope prof(0, stream);

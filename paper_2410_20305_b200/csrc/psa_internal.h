@@ -43,6 +43,7 @@ struct PlanPart {
   int32_t q_tile0 = 0, n_q_tiles = 0;    // query tiles
   int32_t cta0 = 0, n_ctas = 0;          // (key tile, kv head) pairs of the backward's launch order
   int32_t few0 = 0, n_few = 0;           // few-key rows
+  int32_t fwd_items_per_cta = 2;         // work items (query tile, query head) that a CTA of the forward takes: 1 or 2
   int32_t bwd_split = 1;                 // CTAs (a cluster) that share the iterations of one such pair: 1, 2, 4 or 8
 };
 

@@ -63,6 +63,23 @@ bool precise_rows(int i, int len, int cs, int rs) {
   return q < q1 && cs + (q - rs + 1) < kTile;       // it sees the prompt and q - rs + 1 own keys
 }
 
+// Work items that a CTA of the forward takes.  Two pay the CTA's fixed costs once for both; one each spreads the items
+// over more of the CTAs that the chip holds at a time (two per SM), and a launch lasts at least as long as its longest
+// CTA.  In key tiles, with 4 for an item's fixed costs: two, where the share of a resident CTA is at least 92 % of two
+// longest items.  Of 134 packs (long prompts, short samples, one sample; 8 to 32 heads of 64 and 128; 160 to 1584 items)
+// the rule is 0.1 % and at most 3.8 % behind the better of the two.  us with one / two:
+//   3876 tokens, 32/8 heads of 128, lists of 2.5 (1152 items) 43.8 / 40.6    8158, 16 of 64, 2.8 (1136) 36.7 / 32.6
+//   858 tokens, 32/8 of 128, 2.6 (256) 14.0 / 21.4           7763, 8/2 of 128, lists of 1 to 24 (496) 48.3 / 82.4
+//   16629, 8/2 of 128, 1 to 36 (1080) 100.1 / 129.0    21996, 8/2 of 128, 1 to 32 (1416) 114.8 / 124.2
+//   5061, 32/8 of 128 (1312) 100.4 / 96.6              31041, 32/8 of 128 (7904) 1019 / 965
+void items_per_cta(const psa_plan_t* p, int n_sm, PlanPart* part) {
+  if (part->n_q_tiles == 0) return;
+  const TileRec* tiles = p->q_tiles.data() + part->q_tile0;
+  int64_t work = 0;
+  for (int32_t i = 0; i < part->n_q_tiles; ++i) work += (tiles[i].list_cnt + 4) * int64_t(p->Hq);
+  part->fwd_items_per_cta = work * 100 >= 92 * 2 * int64_t(n_sm) * (2 * int64_t(tiles[0].list_cnt + 4)) ? 2 : 1;
+}
+
 // Launch order of the backward for the samples [s0, s1), appended to the plan's list, and the number of CTAs that share
 // the iterations of one (key tile, kv head) pair.
 //
@@ -266,6 +283,7 @@ extern "C" psa_status_t psa_plan(const int32_t* cu_seqlens, const int32_t* prefi
     p->whole.row1 = p->T;
     p->whole.n_q_tiles = int32_t(p->q_tiles.size());
     p->whole.n_few = int32_t(p->few_key_rows.size());
+    psa::items_per_cta(p, n_sm, &p->whole);
     psa::order_backward(p, tiles_of, 0, n_samples, n_sm, &p->whole);
 
     // Parts for psa_step_host: runs of whole samples of about a sixth of the pack (4 to 24 differ by 5 %; with more
@@ -292,6 +310,7 @@ extern "C" psa_status_t psa_plan(const int32_t* cu_seqlens, const int32_t* prefi
         const int32_t n_few = int32_t(p->few_key_rows.size());
         while (w.few0 < n_few && p->few_key_rows[w.few0].row < w.row0) ++w.few0;
         while (w.few0 + w.n_few < n_few && p->few_key_rows[w.few0 + w.n_few].row < w.row1) ++w.n_few;
+        psa::items_per_cta(p, n_sm, &w);
         psa::order_backward(p, tiles_of, first[i], first[i + 1], n_sm, &w);
         p->parts.push_back(w);
       }
@@ -496,6 +515,13 @@ extern "C" psa_status_t psa_plan_counts(const psa_plan_t* p, int32_t direction, 
   const auto& entries = direction ? p->bwd_entries : p->fwd_entries;
   if (n_tiles) *n_tiles = direction ? int32_t(p->kv_tiles.size()) : p->whole.n_q_tiles;
   if (n_entries) *n_entries = int32_t(entries.size());
+  return PSA_OK;
+}
+
+extern "C" psa_status_t psa_plan_launch(const psa_plan_t* p, int32_t* fwd_items_per_cta, int32_t* bwd_ctas_per_pair) {
+  if (!p) return PSA_ERR_INVALID_ARG;
+  if (fwd_items_per_cta) *fwd_items_per_cta = p->whole.fwd_items_per_cta;
+  if (bwd_ctas_per_pair) *bwd_ctas_per_pair = p->whole.bwd_split;
   return PSA_OK;
 }
 
