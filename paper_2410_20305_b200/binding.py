@@ -262,7 +262,7 @@ def psa_bwd(plan: Plan, d_o, q, k, v, o, lse, dq=None, dk=None, dv=None, workspa
     _want_attention(plan, [("d_o", d_o, "q"), ("q", q, "q"), ("k", k, "kv"), ("v", v, "kv"), ("o", o, "q"),
                            ("dq", dq, "q"), ("dk", dk, "kv"), ("dv", dv, "kv")], lse=lse)
     if workspace is None:
-        workspace = torch.empty(max(plan.bwd_workspace_bytes, 256), dtype=torch.uint8, device=q.device)
+        workspace = _temporary(max(plan.bwd_workspace_bytes, 256), torch.uint8, q.device, stream)
     if not workspace.is_cuda or workspace.numel() * workspace.element_size() < plan.bwd_workspace_bytes:
         raise ValueError("workspace: a CUDA buffer of at least %d bytes is needed" % plan.bwd_workspace_bytes)
     _check("psa_bwd", load_library().psa_bwd(plan._h, _ptr(d_o), _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse),
@@ -282,7 +282,7 @@ def psa_bwd_f32(plan: Plan, d_o, q, k, v, o, lse, dq=None, dk=None, dv=None, wor
     _want_attention(plan, [("d_o", d_o, "q"), ("q", q, "q"), ("k", k, "kv"), ("v", v, "kv"), ("o", o, "q")],
                     f32=[("dq", dq, "q"), ("dk", dk, "kv"), ("dv", dv, "kv")], lse=lse)
     if workspace is None:
-        workspace = torch.empty(max(plan.bwd_workspace_bytes, 256), dtype=torch.uint8, device=q.device)
+        workspace = _temporary(max(plan.bwd_workspace_bytes, 256), torch.uint8, q.device, stream)
     if not workspace.is_cuda or workspace.numel() * workspace.element_size() < plan.bwd_workspace_bytes:
         raise ValueError("workspace: a CUDA buffer of at least %d bytes is needed" % plan.bwd_workspace_bytes)
     _check("psa_bwd_f32", load_library().psa_bwd_f32(plan._h, _ptr(d_o), _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse),

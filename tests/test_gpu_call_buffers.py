@@ -8,7 +8,7 @@ from oracle import psa_oracle as orc
 from paper_2410_20305_b200 import binding as B
 from paper_2410_20305_b200 import workloads as wl
 
-from gpu_util import read_status
+from gpu_util import device_plan, max_abs, read_status
 
 pytestmark = pytest.mark.gpu
 
@@ -89,3 +89,28 @@ def test_dpo_logp_scratch_of_the_caller(monkeypatch):
     for small in (scratch[:6], torch.zeros(7, dtype=torch.float64)):
         with pytest.raises(ValueError):
             B.dpo_logp(*args, scratch=small)
+
+
+@pytest.mark.parametrize("name,at", [("psa_bwd", 10), ("psa_bwd_f32", 10)])
+def test_backward_workspace_on_a_stream_that_is_not_current(monkeypatch, name, at):
+    pack = wl.random_pack(6, 3, 300, 4, 2, 64)
+    plan = device_plan(pack)
+    q, k, v, d_o = (t.cuda() for t in wl.attention_inputs(pack, 2))
+    o, lse = B.psa_fwd(plan, q, k, v)
+    grads = [torch.zeros(t.shape, dtype=torch.float32 if name.endswith("f32") else t.dtype, device="cuda") for t in (q, k, v)]
+    want = getattr(B, name)(plan, d_o, q, k, v, o, lse)
+    rec = _Recorder(name)
+    monkeypatch.setattr(B, "load_library", lambda: rec)
+    side = torch.cuda.Stream()
+    a = torch.randn((4096, 4096), device="cuda", dtype=torch.bfloat16)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        for _ in range(40):
+            a @ a                                      # the side stream is busy while the call returns
+    torch.cuda.current_stream().synchronize()
+    getattr(B, name)(plan, d_o, q, k, v, o, lse, *grads, stream=side.cuda_stream)
+    assert rec.calls[-1][at] not in _blocks_of(plan.bwd_workspace_bytes, 4)
+    side.synchronize()
+    assert torch.equal(grads[1], want[1]) and torch.equal(grads[2], want[2])
+    # dq: unordered fp32 adds, rounded to bf16
+    assert max_abs(grads[0], want[0].cpu().double().numpy()) <= 0.0625
