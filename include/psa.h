@@ -267,10 +267,12 @@ psa_status_t psa_bwd_static_scratch(const psa_plan_t* plan, const void* d_o, con
  * memory into the arena, psa_fwd, psa_bwd, and the copies of o, lse, dq, dk, dv back to host
  * memory; a larger pack goes in parts (runs of samples), whose copies in and out run on two
  * streams of the library under the kernels of other parts.  All of it starts behind what
- * `stream` holds at the call, and `stream` ends behind all of it; a call on a capturing stream
- * uses that stream alone.  It does not synchronise: the outputs are valid once the stream has
- * reached the end of the call's work.  Calls on different streams with
- * different arenas overlap (one call's copies with another's kernels).
+ * `stream` holds at the call, and `stream` ends behind all of it.  It does not synchronise: the
+ * outputs are valid once the stream has reached the end of the call's work.  Calls on different
+ * streams with different arenas overlap (one call's copies with another's kernels) and do not
+ * wait for one another: the library keeps two pairs of copy streams per device (created by the
+ * first psa_plan_upload of such a pack), a call takes a pair that no other stream's work is
+ * queued on, and one that finds none, like a call on a capturing stream, uses its own stream alone.
  *   h_q, h_do   host bf16 [T, Hq, d]       h_k, h_v    host bf16 [T, Hkv, d]      (in)
  *   h_o, h_dq   host bf16 [T, Hq, d]       h_dk, h_dv  host bf16 [T, Hkv, d]      (out)
  *   h_lse       host fp32 [Hq, T]                                                (out)

@@ -4,8 +4,6 @@
 #include <cstdio>
 #include <cstdlib>
 #include <mutex>
-#include <new>
-#include <vector>
 
 #include "psa_internal.h"
 
@@ -24,61 +22,80 @@ bool plan_on_current_device(const psa_plan_t* plan) {
 
 namespace psa {
 namespace {
+// Copy streams of psa_step_host.  A pair belongs to one caller's stream at a time: what is enqueued on it waits for that
+// stream, so a call on another stream gets the pair only when both of its streams have run dry, and otherwise another
+// pair or none (it then uses its own stream alone).  So no call waits for another one's stream.
 struct HostPipe {
-  int device = -1;
   cudaStream_t in = nullptr, out = nullptr;   // copies in, copies out
   cudaEvent_t event = nullptr;
-  std::mutex mutex;                            // one call at a time enqueues
-  ~HostPipe() {   // (work that is still enqueued on the streams runs to its end)
-    if (in) cudaStreamDestroy(in);
-    if (out) cudaStreamDestroy(out);
-    if (event) cudaEventDestroy(event);
-  }
+  unsigned long long owner = 0;                // id of the stream of the last call
+  bool taken = false;                          // a call is enqueueing
 };
-constexpr size_t kHostPipesMax = 4;   // idle pipes kept for the next plan
+// Two pairs: steps on two streams overlap each within themselves, and a third one overlaps with them as a whole.
+constexpr int kHostPipes = 2, kDevicesMax = 32;
 std::mutex g_pipe_mutex;
-std::vector<HostPipe*> g_pipes;
+HostPipe g_pipes[kDevicesMax][kHostPipes];
+bool g_pipes_made[kDevicesMax];
 
-// The plan's pipe: taken from the pool, or created, by the plan's first call.  Null if it cannot be had.
-HostPipe* host_pipe_of(const psa_plan_t* plan) {
-  std::lock_guard<std::mutex> lock(plan->used_mutex);
-  if (plan->host_pipe) return static_cast<HostPipe*>(plan->host_pipe);
-  HostPipe* p = nullptr;
-  {
-    std::lock_guard<std::mutex> pool(g_pipe_mutex);
-    for (size_t i = 0; i < g_pipes.size() && !p; ++i)
-      if (g_pipes[i]->device == plan->device) {
-        p = g_pipes[i];
-        g_pipes.erase(g_pipes.begin() + i);
-      }
+// While it lives, a capture in another thread does not mind this thread's calls (none of them touches its streams).
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+bool run_dry(cudaStream_t s) {
+  const cudaError_t e = cudaStreamQuery(s);
+  if (e == cudaErrorNotReady) cudaGetLastError();   // (an answer, not an error of this call)
+  return e == cudaSuccess;
+}
+
+// A pair for one call on `stream`, or null.
+HostPipe* take_host_pipe(int device, cudaStream_t stream) {
+  unsigned long long id = 0;   // (unlike a handle, never given to another stream)
+  if (device >= kDevicesMax) return nullptr;
+  if (cudaStreamGetId(stream, &id) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
   }
-  if (!p) {
-    p = new (std::nothrow) HostPipe;
-    if (!p) return nullptr;
-    p->device = plan->device;
-    if (cudaStreamCreateWithFlags(&p->in, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&p->out, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&p->event, cudaEventDisableTiming) != cudaSuccess) {
-      cudaGetLastError();
-      delete p;
-      return nullptr;
+  std::lock_guard<std::mutex> lock(g_pipe_mutex);
+  RelaxedCapture relaxed;
+  HostPipe* found = nullptr;
+  for (HostPipe& p : g_pipes[device])
+    if (p.event && p.owner == id) {
+      if (p.taken) return nullptr;   // another thread enqueues on the same stream
+      found = &p;
     }
+  for (HostPipe& p : g_pipes[device])
+    if (!found && p.event && !p.taken && run_dry(p.in) && run_dry(p.out)) found = &p;
+  if (found) {
+    found->owner = id;
+    found->taken = true;
   }
-  plan->host_pipe = p;
-  return p;
+  return found;
+}
+
+void give_host_pipe(HostPipe* p) {
+  std::lock_guard<std::mutex> lock(g_pipe_mutex);
+  p->taken = false;
 }
 }  // namespace
 
-void give_host_pipe(void* pipe) {
-  HostPipe* p = static_cast<HostPipe*>(pipe);
-  {
-    std::lock_guard<std::mutex> pool(g_pipe_mutex);
-    if (g_pipes.size() < kHostPipesMax) {
-      g_pipes.push_back(p);
-      return;
-    }
+void make_host_pipes(int device) {
+  std::lock_guard<std::mutex> lock(g_pipe_mutex);
+  if (device < 0 || device >= kDevicesMax || g_pipes_made[device]) return;
+  g_pipes_made[device] = true;
+  RelaxedCapture relaxed;
+  for (HostPipe& p : g_pipes[device]) {
+    if (cudaStreamCreateWithFlags(&p.in, cudaStreamNonBlocking) == cudaSuccess &&
+        cudaStreamCreateWithFlags(&p.out, cudaStreamNonBlocking) == cudaSuccess &&
+        cudaEventCreateWithFlags(&p.event, cudaEventDisableTiming) == cudaSuccess)
+      continue;
+    cudaGetLastError();   // without a pair the calls use their own stream
+    if (p.in) cudaStreamDestroy(p.in);
+    if (p.out) cudaStreamDestroy(p.out);
+    p = HostPipe{};
   }
-  delete p;
 }
 }  // namespace psa
 
@@ -200,7 +217,7 @@ extern "C" psa_status_t psa_step_host(const psa_plan_t* plan, const void* h_q, c
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   psa::HostPipe* pipe = nullptr;
   if (!plan->parts.empty() && cudaStreamIsCapturing(st, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone)
-    pipe = psa::host_pipe_of(plan);
+    pipe = psa::take_host_pipe(plan->device, st);
   if (!pipe) {
     const psa::PlanPart& w = plan->whole;
     if (!copy_in_qkv(w, st) || !copy_in_do(w, st)) return psa::check_last_cuda_error("psa_step_host copy in");
@@ -221,9 +238,7 @@ extern "C" psa_status_t psa_step_host(const psa_plan_t* plan, const void* h_q, c
   // and o leaves under the backward.  7727 tokens, 32/8 heads of 128 (158 MB in, 159 MB out): 6080 -> 4460 us, where
   // the link takes 2870 us for each direction alone and 3670 us for both at once; 3333 tokens of one sample, 8/2
   // heads: 1002 -> 800 us.
-  // An event may be recorded again as soon as the wait for its previous recording has been enqueued; the lock keeps
-  // each such pair together.
-  std::lock_guard<std::mutex> lock(pipe->mutex);
+  // An event may be recorded again as soon as the wait for its previous recording has been enqueued.
   auto order = [&](cudaStream_t before, cudaStream_t after) {
     return cudaEventRecord(pipe->event, before) == cudaSuccess && cudaStreamWaitEvent(after, pipe->event, 0) == cudaSuccess;
   };
@@ -241,6 +256,7 @@ extern "C" psa_status_t psa_step_host(const psa_plan_t* plan, const void* h_q, c
   }
   // The caller's stream ends behind both, also where a part could not be enqueued.
   const bool joined_in = order(pipe->in, st), joined_out = order(pipe->out, st);
+  psa::give_host_pipe(pipe);
   if (rc != PSA_OK) return rc;
   if (!ok || !joined_in || !joined_out) {
     const psa_status_t e = psa::check_last_cuda_error("psa_step_host");

@@ -62,7 +62,6 @@ struct psa_plan {
   // Runs of whole samples for psa_step_host (none for a pack that is not worth splitting).  Where there are several,
   // their query tiles and CTA pairs follow those of the whole pack in q_tiles and bwd_cta_map, in the order of the runs.
   std::vector<psa::PlanPart> parts;
-  mutable void* host_pipe = nullptr;   // psa::HostPipe of psa_step_host, created by its first call
   std::vector<psa::FewKeyRow> few_key_rows;
   // device copy (one allocation, taken from and returned to a small process-wide cache so that a
   // plan per step costs no cudaMalloc / cudaFree and no host synchronisation)
@@ -112,8 +111,8 @@ struct BwdWorkspace {
 };
 BwdWorkspace bwd_workspace_layout(int64_t T, int Hq, int d);
 
-// Hands the streams and events of psa_step_host back to their process-wide pool.
-void give_host_pipe(void* pipe);
+// Creates the copy streams of psa_step_host for a device, once in a process.
+void make_host_pipes(int device);
 
 psa_status_t launch_fwd(const psa_plan_t* plan, const PlanPart& part, const void* q, const void* k, const void* v, void* o,
                         float* lse, int32_t* device_status, void* stream);

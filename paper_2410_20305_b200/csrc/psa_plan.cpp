@@ -407,6 +407,7 @@ extern "C" psa_status_t psa_plan_upload(psa_plan_t* p, void* stream) {
   const size_t b5 = up(p->few_key_rows.size() * sizeof(psa::FewKeyRow));
   const size_t total = b0 + b1 + b2 + b3 + b4 + b5 + 256;
   if (cudaGetDevice(&p->device) != cudaSuccess) return PSA_ERR_CUDA;
+  if (!p->parts.empty()) psa::make_host_pipes(p->device);   // here, so that psa_step_host creates nothing
   BlobEntry e;
   if (!take_entry(p->device, total, &e)) return PSA_ERR_CUDA;
   const cudaStream_t st = cudaStream_t(stream);
@@ -492,7 +493,6 @@ extern "C" psa_status_t psa_plan_destroy(psa_plan_t* p) {
     if (cur >= 0 && cur != p->device) cudaSetDevice(cur);
     give_entry(e);
   }
-  if (p->host_pipe) psa::give_host_pipe(p->host_pipe);
   delete p;
   return st;
 }

@@ -99,3 +99,64 @@ def test_step_host_in_parts_equals_the_device_calls(lengths, heads):
         assert torch.equal(out[3], grads[1].cpu()) and torch.equal(out[4], grads[2].cpu())
         want = grads[0].cpu().double()          # dq: unordered fp32 adds, rounded to bf16
         assert ((out[2].double() - want).abs() <= 2.0 ** -7 * want.abs() + 1e-4).all()
+
+
+def _host_set(pack, seed, plan):
+    t = [x.pin_memory() for x in wl.attention_inputs(pack, seed)]
+    q, k = t[0], t[1]
+    out = [torch.zeros_like(q).pin_memory(), torch.zeros((q.shape[1], q.shape[0])).pin_memory(),
+           torch.zeros_like(q).pin_memory(), torch.zeros_like(k).pin_memory(), torch.zeros_like(k).pin_memory()]
+    return t, out, torch.empty(B.psa_step_host_arena_bytes(plan), dtype=torch.uint8, device="cuda")
+
+
+def _same_as_device_calls(plan, t, out):
+    q, k, v, d_o = (x.cuda() for x in t)
+    o, lse = B.psa_fwd(plan, q, k, v)
+    grads = B.psa_bwd(plan, d_o, q, k, v, o, lse)
+    assert torch.equal(out[0], o.cpu()) and torch.equal(out[1], lse.cpu())
+    assert torch.equal(out[3], grads[1].cpu()) and torch.equal(out[4], grads[2].cpu())
+    want = grads[0].cpu().double()          # dq: unordered fp32 adds, rounded to bf16
+    assert ((out[2].double() - want).abs() <= 2.0 ** -7 * want.abs() + 1e-4).all()
+
+
+PARTS = wl.pack_from_lengths("parts", [(700, 80, 90), (300, 200, 100), (50, 60, 70)] * 2, 32, 8, 64)
+
+
+def test_a_call_does_not_wait_for_another_stream():
+    """The first call's stream is busy; a second call of the same plan, and one of another plan, on idle streams come
+    back before that stream has got to the first."""
+    plans = [device_plan(PARTS), device_plan(PARTS)]
+    sets = [_host_set(PARTS, seed, plans[0]) for seed in (1, 2, 3, 4)]
+    busy, idle, third = (torch.cuda.Stream() for _ in range(3))
+    a = torch.randn((8192, 8192), device="cuda", dtype=torch.bfloat16)
+    b = torch.empty_like(a)
+    for plan, stream, (t, out, arena) in ((plans[0], idle, sets[1]), (plans[1], third, sets[2])):   # (once, as warm-up)
+        B.psa_step_host(plan, *t, *out, arena, stream=stream.cuda_stream)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(busy):
+        for _ in range(400):
+            torch.mm(a, a, out=b)
+        passed = torch.cuda.Event()
+        passed.record()
+    for plan, stream, (t, out, arena) in ((plans[0], busy, sets[0]), (plans[0], idle, sets[1]), (plans[1], third, sets[2]),
+                                          (plans[0], idle, sets[3])):
+        B.psa_step_host(plan, *t, *out, arena, stream=stream.cuda_stream)
+    idle.synchronize()
+    third.synchronize()
+    assert not passed.query()
+    torch.cuda.synchronize()
+    for t, out, _ in sets:
+        _same_as_device_calls(plans[0], t, out)
+
+
+def test_many_streams_and_plans_at_once():
+    plans = [device_plan(PARTS) for _ in range(3)]
+    sets = [_host_set(PARTS, seed, plans[0]) for seed in range(4)]
+    streams = [torch.cuda.Stream() for _ in range(4)]
+    torch.cuda.synchronize()
+    for i in range(24):
+        t, out, arena = sets[i % 4]
+        B.psa_step_host(plans[i % 3], *t, *out, arena, stream=streams[i % 4].cuda_stream)
+    torch.cuda.synchronize()
+    for t, out, _ in sets:
+        _same_as_device_calls(plans[0], t, out)
