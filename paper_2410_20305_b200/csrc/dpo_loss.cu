@@ -281,7 +281,7 @@ dpo_logp_bwd_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_str
   extern __shared__ __align__(16) uint4 s_row[];   // kStaged: the whole vectors of the row
   __shared__ __align__(8) uint64_t s_bar[kParts];
   __shared__ float2 s_part[kThreads / 32];
-  __shared__ int s_abort;
+  __shared__ int s_abort, s_late;
   const int64_t row = blockIdx.x;
   const int tid = threadIdx.x;
   const T* x = logits + row * row_stride;
@@ -307,7 +307,7 @@ dpo_logp_bwd_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_str
     const int part = (n + kParts * kThreads - 1) / (kParts * kThreads) * kThreads;   // whole turns of the block
     const uint32_t bar0 = dev::smem_u32(s_bar);
     if (tid == 0) {
-      s_abort = 0;
+      s_abort = s_late = 0;
       for (int p = 0; p < kParts; ++p) dev::mbar_init(bar0 + 8 * p, 1);
       dev::fence_mbar_init();
       for (int p = 0; p < kParts; ++p) {
@@ -330,6 +330,16 @@ dpo_logp_bwd_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_str
   }
   for (int64_t j = n_vec * E + tid; j < vocab; j += kThreads) acc.merge(Elem<T>::load1(x + j) * kLog2e, 1.f);
   const float lse2 = block_lse2<kThreads>(acc, s_part);
+  if constexpr (kStaged) {
+    if (*static_cast<volatile int*>(&s_abort)) {
+      // A wait has expired (and said so): the row is not written, and the CTA stays until the copies into its shared
+      // memory have ended, again for a limited time.
+      const dev::WaitCtx again{&s_late, status, dev::kWaitLimitClocks};
+      const int n = int(n_vec), part = (n + kParts * kThreads - 1) / (kParts * kThreads) * kThreads;
+      for (int p = 0; tid == 0 && p < kParts && p * part < n; ++p) dev::mbar_wait(dev::smem_u32(s_bar) + 8 * p, 0, again);
+      return;
+    }
+  }
 
   if constexpr (kStaged) {
     for (int i = tid; i < int(n_vec); i += kThreads) st_stream(dv + i, grad_vector<T>(s_row[i], lab.csum, lse2));
