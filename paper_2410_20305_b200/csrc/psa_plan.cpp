@@ -66,8 +66,10 @@ bool precise_rows(int i, int len, int cs, int rs) {
 // Work items that a CTA of the forward takes.  Two pay the CTA's fixed costs once for both; one each spreads the items
 // over more of the CTAs that the chip holds at a time (two per SM), and a launch lasts at least as long as its longest
 // CTA.  In key tiles, with 4 for an item's fixed costs: two, where the share of a resident CTA is at least 92 % of two
-// longest items.  Of 134 packs (long prompts, short samples, one sample; 8 to 32 heads of 64 and 128; 160 to 1584 items)
-// the rule is 0.1 % and at most 3.8 % behind the better of the two.  us with one / two:
+// longest items.  Over 300 packs drawn from long prompts, short samples, single samples (450 to 2400 items) the rule is
+// 0.15 % behind the better of the two, more than 2 % in 8 of them and 7 % in one; a line at 1184 items is 0.56 % behind,
+// more than 2 % in 27 and 13 % in one.  (A simulation of both launches: 0.10 %, more than 2 % in 6; not worth its time.)
+// us with one / two:
 //   3876 tokens, 32/8 heads of 128, lists of 2.5 (1152 items) 43.8 / 40.6    8158, 16 of 64, 2.8 (1136) 36.7 / 32.6
 //   858 tokens, 32/8 of 128, 2.6 (256) 14.0 / 21.4           7763, 8/2 of 128, lists of 1 to 24 (496) 48.3 / 82.4
 //   16629, 8/2 of 128, 1 to 36 (1080) 100.1 / 129.0    21996, 8/2 of 128, 1 to 32 (1416) 114.8 / 124.2
