@@ -184,3 +184,46 @@ def test_terms_at_the_ends_of_their_range(dtype, vocab):
     # (vocab 1: log2 of a sum that should be 1, with the exponential's error)
     assert abs(got[3] - want[3]) <= 1e-6 * 4 * 10 + 6e-8 * abs(want[3]), (got[3], want[3])
     assert got[4] == 0 and (got[[0, 3]] <= 0).all()
+
+
+@pytest.mark.parametrize("dtype,vocab", [(torch.float32, 1001), (torch.bfloat16, 1003), (torch.bfloat16, 33000), (torch.float32, 17000)])
+def test_the_entry_point_without_scratch(dtype, vocab):
+    """dpo_logp of the C ABI: fp32 sums added straight into out."""
+    rows, stride = 300, (vocab + 7) // 8 * 8
+    x, _ = wl.logits_and_tokens(rows, stride, 6, 3.0 ** 0.5, dtype)
+    rng = np.random.default_rng(3)
+    targets = rng.integers(0, vocab, rows).astype(np.int32)
+    seg = rng.integers(-1, 4, rows).astype(np.int32)
+    forks = [np.array(a, dtype=np.int32) for a in ([0, 299, 7], [vocab - 1, 0, 5], [3, 0, 1])]
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = torch.full((5,), 7.0, device="cuda")
+    xd, dev = x.cuda(), [_dev(a) for a in (targets, seg, *forks)]
+    code = B.load_library().dpo_logp(xd.data_ptr(), B.PSA_DTYPE_F32 if dtype == torch.float32 else B.PSA_DTYPE_BF16, rows, vocab,
+                                     stride, *(a.data_ptr() for a in dev), 3, 4, out.data_ptr(), status.data_ptr(),
+                                     torch.cuda.current_stream().cuda_stream)
+    assert code == 0 and read_status(status) == 0
+    want = orc.dpo_logp(wl.to_f64(x)[:, :vocab], targets, seg, 4, *forks)
+    got = out.cpu().double().numpy()
+    # per term an ulp of its fp32 log-sum-exp, and half an ulp of the running sum (6e-8 of it) for each of about 60 terms
+    assert got[4] == 7.0 and (np.abs(got[:4] - want) <= 300 * 1e-6 + 60 * 6e-8 * np.abs(want)).all()
+
+
+def test_a_captured_call_is_replayed_with_new_logits():
+    rows, vocab = 200, 1000
+    rng = np.random.default_rng(8)
+    targets, seg = rng.integers(0, vocab, rows).astype(np.int32), rng.integers(-1, 6, rows).astype(np.int32)
+    x = torch.zeros((rows, vocab), dtype=torch.bfloat16, device="cuda")
+    args = x, _dev(targets), _dev(seg), 6
+    out = torch.zeros(6, device="cuda")
+    B.dpo_logp(*args, out=out)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        B.dpo_logp(*args, out=out)
+    for seed in (1, 2):
+        new, _ = wl.logits_and_tokens(rows, vocab, seed, 3.0 ** 0.5, torch.bfloat16)
+        x.copy_(new)
+        graph.replay()
+        torch.cuda.synchronize()
+        want = orc.dpo_logp(wl.to_f64(new), targets, seg, 6)
+        assert (np.abs(out.cpu().double().numpy() - want) <= TOL_LOGP * np.abs(want)).all()

@@ -101,11 +101,12 @@ def test_step_host_in_parts_equals_the_device_calls(lengths, heads):
         assert ((out[2].double() - want).abs() <= 2.0 ** -7 * want.abs() + 1e-4).all()
 
 
-def _host_set(pack, seed, plan):
-    t = [x.pin_memory() for x in wl.attention_inputs(pack, seed)]
+def _host_set(pack, seed, plan, pinned=True):
+    place = lambda x: x.pin_memory() if pinned else x.clone()  # noqa: E731
+    t = [place(x) for x in wl.attention_inputs(pack, seed)]
     q, k = t[0], t[1]
-    out = [torch.zeros_like(q).pin_memory(), torch.zeros((q.shape[1], q.shape[0])).pin_memory(),
-           torch.zeros_like(q).pin_memory(), torch.zeros_like(k).pin_memory(), torch.zeros_like(k).pin_memory()]
+    out = [place(x) for x in (torch.zeros_like(q), torch.zeros((q.shape[1], q.shape[0])), torch.zeros_like(q),
+                              torch.zeros_like(k), torch.zeros_like(k))]
     return t, out, torch.empty(B.psa_step_host_arena_bytes(plan), dtype=torch.uint8, device="cuda")
 
 
@@ -160,3 +161,38 @@ def test_many_streams_and_plans_at_once():
     torch.cuda.synchronize()
     for t, out, _ in sets:
         _same_as_device_calls(plans[0], t, out)
+
+
+@pytest.mark.parametrize("lengths,heads", [([(700, 80, 90), (300, 200, 100), (50, 60, 70)] * 2, (32, 8, 64)),
+                                           ([(900, 100, 100)], (16, 16, 128))])
+def test_pageable_host_buffers_in_parts(lengths, heads):
+    pack = wl.pack_from_lengths("parts", lengths, *heads)
+    assert pack.total_tokens * heads[0] * heads[2] * 2 > 2 << 20
+    plan = device_plan(pack)
+    t, out, arena = _host_set(pack, 5, plan, pinned=False)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    B.psa_step_host(plan, *t, *out, arena, stream=stream.cuda_stream)
+    stream.synchronize()
+    _same_as_device_calls(plan, t, out)
+
+
+def test_a_captured_call_is_replayed_with_new_inputs():
+    """A call on a capturing stream uses that stream alone; each replay copies what the host buffers then hold."""
+    plan = device_plan(PARTS)
+    t, out, arena = _host_set(PARTS, 6, plan)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    B.psa_step_host(plan, *t, *out, arena, stream=stream.cuda_stream)   # (the plan has been used on the stream before)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        B.psa_step_host(plan, *t, *out, arena)
+    for seed in (7, 8):
+        for x, y in zip(t, wl.attention_inputs(PARTS, seed)):
+            x.copy_(y)
+        for x in out:
+            x.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        _same_as_device_calls(plan, t, out)
