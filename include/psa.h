@@ -321,7 +321,8 @@ psa_status_t dpo_logp(const void* logits, int32_t logits_dtype, int64_t n_rows, 
                       float* out, int32_t* device_status, void* stream);
 
 /*
- * dpo_logp_f64sum -- dpo_logp with the sums of the responses taken in fp64 and rounded once.
+ * dpo_logp_f64sum -- dpo_logp with the sums of the responses taken in fp64 and rounded once (a term
+ * that rounding has put above 0 counts as 0).
  *   scratch   device memory of 8 * (n_segments + 1) bytes, 8-byte aligned; contents on entry are
  *             ignored, on exit undefined
  * Everything else, and the errors, as dpo_logp.

@@ -224,7 +224,7 @@ psa_status_t run_logp(const void* logits, int32_t logits_dtype, int64_t n_rows, 
   // the stride is not used when there is a single row
   if ((reinterpret_cast<uintptr_t>(logits) & 15) || (n_rows > 1 && ((row_stride * esz) & 15))) return PSA_ERR_ALIGNMENT;
   cudaStream_t st = cudaStream_t(stream);
-  if (n_rows == 0) sums = nullptr;   // nothing runs that would round them
+  if (n_rows == 0) sums = nullptr;   // nothing is added: only out is cleared
   if (sums && n_segments > 0)
     psa::dpo_logp_clear_kernel<<<unsigned(n_segments + 127) / 128, 128, 0, st>>>(out, sums, n_segments);
   else if (n_segments > 0 && cudaMemsetAsync(out, 0, sizeof(float) * size_t(n_segments), st) != cudaSuccess)
@@ -238,7 +238,8 @@ psa_status_t run_logp(const void* logits, int32_t logits_dtype, int64_t n_rows, 
   // Threads x loads in flight per thread.  Small CTAs keep many rows in flight per SM and retire unevenly, which suits
   // many rows: 16215 x 128256 bf16, 2/3 live, 400 us with 128 x 4, 408 with 256 x 4, 484 with 512 x 4.  A few long rows
   // are less than two waves of 1480 such CTAs, and a wave lasts as long as a row: 1800 x 128256 bf16 66 -> 60 us with
-  // 256 x 4.  fp32 rows have half the exponentials per byte and take more loads in flight from 64 KB on: 4096 x 50257
+  // 256 x 4.  (The host knows the number of rows, not how many of them are live: a frozen model's pass with 1200 live of
+  // 15154 rows is such a launch too, but takes 128 x 4.)  fp32 rows have half the exponentials per byte and take more loads in flight from 64 KB on: 4096 x 50257
   // 107 -> 85 us with 256 x 8, 8192 x 50257 171 -> 157, 4000 x 16384 36 -> 33, 3312 x 115288 (360 live) 54 -> 37; below,
   // 128 x 4 stays better (6000 x 8192 27 against 29).
   const int64_t row_bytes = vocab * esz;

@@ -2,8 +2,9 @@
 // read as  -log sigmoid(beta * [(lp_theta(c) - lp_ref(c)) - (lp_theta(r) - lp_ref(r))]),
 // averaged over the samples) and its gradient back into the logits,
 //     dlogits[t][v] = sum over labels (t, y, g) scored by row t of  coef[g] * (1[v == y] - softmax(logits[t])[v]).
-// dpo_logp_bwd is HBM-bound: every live row is read once from DRAM (the second sweep reads it from shared memory or
-// L2) and written once with streaming stores; rows that score nothing are only written (zeros).
+// dpo_logp_bwd is HBM-bound: a live row is read for two sweeps, the second from shared memory (rows up to 96 KB: one
+// read from DRAM) or from L2, where not all of it is left (1000 x 128256 bf16: 17 % of the live bytes come from DRAM a
+// second time), and written once with streaming stores; rows that score nothing are only written (zeros).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>

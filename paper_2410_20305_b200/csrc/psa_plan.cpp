@@ -65,9 +65,9 @@ bool precise_rows(int i, int len, int cs, int rs) {
 
 // Work items that a CTA of the forward takes.  Two pay the CTA's fixed costs once for both; one each spreads the items
 // over more of the CTAs that the chip holds at a time (two per SM), and a launch lasts at least as long as its longest
-// CTA.  In key tiles, with 4 for an item's fixed costs: two, where the share of a resident CTA is at least 92 % of two
+// CTA.  In key tiles, with 3.5 for an item's fixed costs: two, where the share of a resident CTA is at least 94 % of two
 // longest items.  Over 300 packs drawn from long prompts, short samples, single samples (450 to 2400 items) the rule is
-// 0.15 % behind the better of the two, more than 2 % in 8 of them and 7 % in one; a line at 1184 items is 0.56 % behind,
+// 0.18 % behind the better of the two, more than 2 % in 11 of them and 7 % in one; a line at 1184 items is 0.56 % behind,
 // more than 2 % in 27 and 13 % in one.  (A simulation of both launches: 0.10 %, more than 2 % in 6; not worth its time.)
 // us with one / two:
 //   3876 tokens, 32/8 heads of 128, lists of 2.5 (1152 items) 43.8 / 40.6    8158, 16 of 64, 2.8 (1136) 36.7 / 32.6
@@ -78,8 +78,9 @@ void items_per_cta(const psa_plan_t* p, int n_sm, PlanPart* part) {
   if (part->n_q_tiles == 0) return;
   const TileRec* tiles = p->q_tiles.data() + part->q_tile0;
   int64_t work = 0;
-  for (int32_t i = 0; i < part->n_q_tiles; ++i) work += (tiles[i].list_cnt + 4) * int64_t(p->Hq);
-  part->fwd_items_per_cta = work * 100 >= 92 * 2 * int64_t(n_sm) * (2 * int64_t(tiles[0].list_cnt + 4)) ? 2 : 1;
+  for (int32_t i = 0; i < part->n_q_tiles; ++i) work += (2 * tiles[i].list_cnt + 7) * int64_t(p->Hq);
+  const int64_t two_longest = 2 * (2 * int64_t(tiles[0].list_cnt) + 7);
+  part->fwd_items_per_cta = work * 100 >= 94 * 2 * int64_t(n_sm) * two_longest ? 2 : 1;
 }
 
 // Launch order of the backward for the samples [s0, s1), appended to the plan's list, and the number of CTAs that share
