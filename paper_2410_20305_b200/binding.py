@@ -332,7 +332,7 @@ def dpo_logp(logits, targets, segment_ids, n_segments, fork_rows=None, fork_targ
     if out is None:
         out = torch.empty(n_segments, dtype=torch.float32, device=logits.device)
     if scratch is None:
-        scratch = _temporary(n_segments + 1, torch.float64, logits.device, stream)
+        scratch = _temporary(max(n_segments, 0) + 1, torch.float64, logits.device, stream)
     elif not scratch.is_cuda or scratch.numel() * scratch.element_size() < 8 * (n_segments + 1):
         raise ValueError("scratch: a CUDA buffer of at least %d bytes is needed" % (8 * (n_segments + 1)))
     _check("dpo_logp", load_library().dpo_logp_f64sum(

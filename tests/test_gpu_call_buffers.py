@@ -91,6 +91,14 @@ def test_dpo_logp_scratch_of_the_caller(monkeypatch):
             B.dpo_logp(*args, scratch=small)
 
 
+@pytest.mark.parametrize("n_segments", [-1, -2, -100])
+def test_a_negative_number_of_responses_is_refused_by_the_library(n_segments):
+    (x, targets, seg, _), _ = _logp_inputs(8, 64, 2, 5)
+    with pytest.raises(B.PsaError) as e:
+        B.dpo_logp(x, targets, seg, n_segments, out=torch.zeros(2, device="cuda"))
+    assert e.value.code == 1
+
+
 @pytest.mark.parametrize("name,at", [("psa_bwd", 10), ("psa_bwd_f32", 10)])
 def test_backward_workspace_on_a_stream_that_is_not_current(monkeypatch, name, at):
     pack = wl.random_pack(6, 3, 300, 4, 2, 64)
