@@ -170,10 +170,8 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 
   // Iteration it (of this CTA) -> (query head of the group, entry of the list).
   auto head_of = [&](int it) { return hk * g + (kSplit ? it0 + it : it) / n_list; };
-  auto entry_of = [&](int it) {
-    const int li = (kSplit ? it0 + it : it) % n_list;
-    return li < L::kEntCap ? s_ent[li] : ent[li];
-  };
+  auto entry_at = [&](int li) { return li < L::kEntCap ? s_ent[li] : ent[li]; };
+  auto entry_of = [&](int it) { return entry_at((kSplit ? it0 + it : it) % n_list); };
 
   // Each warpgroup changes its register budget as its first action, inside its own branch, so
   // that everything the branch executes afterwards is compiled for that budget.
@@ -315,19 +313,29 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     const int qend = (kv_local >= rec.cs && kv_local < rec.rs) ? rec.rs : rec.len;
     const float cl = prm.scale_log2;
 
-    // Per-column statistics of the iteration's query tile: workers 0..127 fetch lse * log2e,
-    // workers 128..255 fetch delta, each for column (wt & 127).
-    auto load_stat = [&](int it) {
-      const int64_t qrow = int64_t(rec.ds) + (entry_of(it) >> 2) * kTile + (wt & 127);
+    // Per-column statistics of an iteration's query tile: workers 0..127 fetch lse, workers 128..255 fetch delta, each
+    // for column (wt & 127).  They are asked for an iteration ahead and first touched (scaled, stored) at its end: with
+    // the scaling beside the load, and divisions to find the next query head and list position, the workers stood still
+    // for 1200 of an iteration's 3600 clocks at head size 64.  us of the backward: 20774 tokens, 16 heads of 64, 500 ->
+    // 471; 7965 tokens, 16 of 64, fp32 gradients, 131 -> 126; 7727 tokens, 32/8 of 128, 221 -> 215; long lists at 128
+    // are paced by the other roles (31041 tokens 2435 -> 2424, one sample of 16700 1413 -> 1430).
+    const float* const stat_of = wt < 128 ? prm.lse : prm.delta;
+    const float stat_mul = wt < 128 ? kLog2e : 1.f;
+    auto load_stat = [&](int h, int e) {
+      const int64_t qrow = int64_t(rec.ds) + (e >> 2) * kTile + (wt & 127), idx = int64_t(h) * prm.T + qrow;
       float x = 0.f;
-      if (qrow < prm.row_end && PSA_IN_BOUNDS(int64_t(head_of(it)) * prm.T + qrow, int64_t(prm.Hq) * prm.T, prm.status)) {
-        const int64_t idx = int64_t(head_of(it)) * prm.T + qrow;
-        x = wt < 128 ? prm.lse[idx] * kLog2e : prm.delta[idx];
-      }
+      if (qrow < prm.row_end && PSA_IN_BOUNDS(idx, int64_t(prm.Hq) * prm.T, prm.status)) x = stat_of[idx];
       return x;
     };
-    auto store_stat = [&](int st, float x) { (wt < 128 ? s_lse : s_delta)[st * kTile + (wt & 127)] = x; };
-    if (!kSplit || n_it > 0) store_stat(0, load_stat(0));
+    auto store_stat = [&](int st, float x) { (wt < 128 ? s_lse : s_delta)[st * kTile + (wt & 127)] = x * stat_mul; };
+    // Query head, list position and entry of the current iteration.
+    int h_cur = 0, li_cur = 0, e_cur = 0;
+    if (!kSplit || n_it > 0) {
+      h_cur = head_of(0);
+      li_cur = kSplit ? it0 % n_list : 0;
+      e_cur = entry_at(li_cur);
+      store_stat(0, load_stat(h_cur, e_cur));
+    }
     named_bar_sync(1, 256);
 
     uint32_t dse_ph = 0;  // running parity of B_DS_EMPTY
@@ -338,10 +346,17 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     auto iteration = [&](int it, auto precise_tag) {
       constexpr bool kPrecise = decltype(precise_tag)::value;
       const int st = it & 1;
-      const int e = entry_of(it);
+      const int e = e_cur;
       const int q0 = (e >> 2) * kTile;
       float next_stat = 0.f;
-      if (it + 1 < n_it) next_stat = load_stat(it + 1);
+      if (it + 1 < n_it) {
+        if (++li_cur == n_list) {
+          li_cur = 0;
+          ++h_cur;
+        }
+        e_cur = entry_at(li_cur);
+        next_stat = load_stat(h_cur, e_cur);
+      }
 
       mbar_wait(bar(B_S_FULL), it & 1, wctx);
       tc_fence_after();
@@ -491,11 +506,18 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       named_bar_sync(1, 256);
     };
     for (int it = 0; it < n_it; ++it) {
-      if (entry_of(it) & 2) iteration(it, std::true_type{});
+      if (e_cur & 2) iteration(it, std::true_type{});
       else iteration(it, std::false_type{});
     }
-    mbar_wait(bar(B_DONE), 0, wctx);
+    // dV is final before the last dK and dQ are: without a cluster it leaves while these run (7965 tokens, 16 heads of
+    // 64: 126 -> 124 us; at 128 0.2 % of short packs).
+    if constexpr (kSplit) mbar_wait(bar(B_DONE), 0, wctx);
+    else mbar_wait(bar(B_DO_EMPTY), (n_it - 1) & 1, wctx);
     tc_fence_after();
+    auto before_dk = [&]() {
+      mbar_wait(bar(B_DONE), 0, wctx);
+      tc_fence_after();
+    };
 
     // ---- epilogue: this half's columns of dV and dK (scaled) -> bf16, or fp32 as they are
     if constexpr (kSplit) {
@@ -579,6 +601,7 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       const int64_t row = int64_t(rec.row0) + r;
 #pragma unroll
       for (int which = 0; which < 2; ++which) {
+        if (which) before_dk();
         const float mul = which ? prm.scale : 1.f;
         float* dst_row = static_cast<float*>(which ? prm.dk : prm.dv) + (row * prm.Hkv + hk) * D + half * DH;
 #pragma unroll
@@ -602,8 +625,9 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       // box would cover: it takes the per-thread path below.)
 #pragma unroll
       for (int which = 0; which < 2; ++which) {
+        if (which) before_dk();
         const float mul = which ? prm.scale : 1.f;
-        const uint32_t tile = which ? sK : sV;     // dK leaves through the K buffer, dV through V's
+        const uint32_t tile = which ? sK : sV;     // dK leaves through the K buffer, dV through V's (no longer read)
 #pragma unroll
         for (int ch = 0; ch < DH / 32; ++ch) {
           uint32_t v[32];
@@ -621,23 +645,21 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                          pack_bf16x2(__uint_as_float(v[8 * i + 6]) * mul, __uint_as_float(v[8 * i + 7]) * mul));
           }
         }
-      }
-      fence_proxy_async_smem();
-      named_bar_sync(1, 256);
-      if (leader) {
-        for (int s = 0; s < L::kSub; ++s) {
-          tma_store_3d(&tm_dv, sV + s * L::kSubBytes, s * 64, hk, rec.row0);
-          tma_store_3d(&tm_dk, sK + s * L::kSubBytes, s * 64, hk, rec.row0);
+        fence_proxy_async_smem();
+        named_bar_sync(1, 256);
+        if (leader) {
+          for (int s = 0; s < L::kSub; ++s) tma_store_3d(which ? &tm_dk : &tm_dv, tile + s * L::kSubBytes, s * 64, hk, rec.row0);
+          tma_commit_group();
         }
-        tma_commit_group();
-        tma_wait_group_read<0>();   // shared memory must outlive the stores' reads
       }
+      if (leader) tma_wait_group_read<0>();   // shared memory must outlive the stores' reads
     } else {
     const int64_t row = int64_t(rec.row0) + r;
     __nv_bfloat16* dv_row = static_cast<__nv_bfloat16*>(prm.dv) + (row * prm.Hkv + hk) * D + half * DH;
     __nv_bfloat16* dk_row = static_cast<__nv_bfloat16*>(prm.dk) + (row * prm.Hkv + hk) * D + half * DH;
 #pragma unroll
     for (int which = 0; which < 2; ++which) {
+      if (which) before_dk();
       const float mul = which ? prm.scale : 1.f;
       __nv_bfloat16* dst_row = which ? dk_row : dv_row;
 #pragma unroll
