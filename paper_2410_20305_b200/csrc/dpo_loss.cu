@@ -14,6 +14,7 @@
 #include "psa.h"
 #include "psa_device.cuh"
 #include "psa_internal.h"
+#include "psa_launch.cuh"
 
 namespace psa {
 namespace {
@@ -86,6 +87,7 @@ struct MaxSum {
 __global__ void dpo_loss_kernel(const float* __restrict__ pol, const float* __restrict__ ref, int n, float beta,
                                 float* __restrict__ loss, float* __restrict__ coef) {
   __shared__ float part[32];
+  behind_wait();
   float acc = 0.f;
   for (int s = threadIdx.x; s < n; s += blockDim.x) {
     const float z = beta * ((pol[2 * s] - ref[2 * s]) - (pol[2 * s + 1] - ref[2 * s + 1]));
@@ -110,6 +112,7 @@ __global__ void simpo_loss_kernel(const float* __restrict__ pol, const int32_t* 
                                   float gamma, float* __restrict__ loss, float* __restrict__ coef,
                                   int32_t* __restrict__ status) {
   __shared__ float part[32];
+  behind_wait();
   float acc = 0.f;
   for (int s = threadIdx.x; s < n; s += blockDim.x) {
     const int lc = len[2 * s], lr = len[2 * s + 1];
@@ -140,6 +143,7 @@ __global__ void simpo_loss_kernel(const float* __restrict__ pol, const int32_t* 
 __global__ void orpo_loss_kernel(const float* __restrict__ pol, const int32_t* __restrict__ len, int n, float lam,
                                  float* __restrict__ loss, float* __restrict__ coef, int32_t* __restrict__ status) {
   __shared__ float part[32];
+  behind_wait();
   float acc = 0.f;
   for (int s = threadIdx.x; s < n; s += blockDim.x) {
     const int lc = len[2 * s], lr = len[2 * s + 1];
@@ -290,6 +294,7 @@ dpo_logp_bwd_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_str
   const uint4* xv = reinterpret_cast<const uint4*>(x);
   uint4* dv = reinterpret_cast<uint4*>(dx);
   const int64_t n_vec = vocab / E;
+  behind_wait();
   const RowLabels lab = row_labels(row, vocab, targets, segment_ids, fork_rows, fork_targets, fork_segments, n_forks,
                                    n_segments, coef, tid == 0, status);
   if (lab.n == 0) {
@@ -385,9 +390,10 @@ psa_status_t launch_logp_bwd(const T* logits, int64_t n_rows, int64_t vocab, int
   if (smem > 40 * 1024 &&
       cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kStagedMost)) != cudaSuccess)
     return PSA_ERR_CUDA;
-  kernel<<<unsigned(n_rows), kThreads, smem, stream>>>(logits, vocab, row_stride, targets, segment_ids, fork_rows,
-                                                      fork_targets, fork_segments, n_forks, n_segments, coef, dlogits,
-                                                      status);
+  // (us of log-probs, loss and gradient with every launch behind the one before: 1515 x 5592 bf16 15.0 -> 13.9, 436 x 2773
+  // fp32 13.1 -> 12.1, 4486 x 4935 bf16 21.1 -> 19.9)
+  launch_behind(true, kernel, dim3(unsigned(n_rows)), kThreads, smem, stream, logits, vocab, row_stride, targets, segment_ids,
+                fork_rows, fork_targets, fork_segments, n_forks, n_segments, coef, dlogits, status);
   return check_last_cuda_error("dpo_logp_bwd launch");
 }
 
@@ -406,14 +412,14 @@ psa_status_t dispatch_logp_bwd(const T* logits, int64_t n_rows, int64_t vocab, A
 extern "C" psa_status_t dpo_loss(const float* policy_logps, const float* ref_logps, int32_t n_samples, float beta,
                                  float* loss, float* coef, void* stream) {
   if (n_samples < 0 || !loss || (n_samples > 0 && (!policy_logps || !ref_logps || !coef))) return PSA_ERR_INVALID_ARG;
-  psa::dpo_loss_kernel<<<1, 256, 0, cudaStream_t(stream)>>>(policy_logps, ref_logps, n_samples, beta, loss, coef);
+  psa::launch_behind(true, psa::dpo_loss_kernel, dim3(1), 256, 0, cudaStream_t(stream), policy_logps, ref_logps, n_samples, beta, loss, coef);
   return psa::check_last_cuda_error("dpo_loss launch");
 }
 
 extern "C" psa_status_t simpo_loss(const float* policy_logps, const int32_t* lengths, int32_t n_samples, float beta,
                                    float gamma, float* loss, float* coef, int32_t* device_status, void* stream) {
   if (n_samples < 0 || !loss || (n_samples > 0 && (!policy_logps || !lengths || !coef))) return PSA_ERR_INVALID_ARG;
-  psa::simpo_loss_kernel<<<1, 256, 0, cudaStream_t(stream)>>>(policy_logps, lengths, n_samples, beta, gamma, loss, coef,
+  psa::launch_behind(true, psa::simpo_loss_kernel, dim3(1), 256, 0, cudaStream_t(stream), policy_logps, lengths, n_samples, beta, gamma, loss, coef,
                                                              device_status);
   return psa::check_last_cuda_error("simpo_loss launch");
 }
@@ -421,7 +427,7 @@ extern "C" psa_status_t simpo_loss(const float* policy_logps, const int32_t* len
 extern "C" psa_status_t orpo_loss(const float* policy_logps, const int32_t* lengths, int32_t n_samples, float lambda,
                                   float* loss, float* coef, int32_t* device_status, void* stream) {
   if (n_samples < 0 || !loss || (n_samples > 0 && (!policy_logps || !lengths || !coef))) return PSA_ERR_INVALID_ARG;
-  psa::orpo_loss_kernel<<<1, 256, 0, cudaStream_t(stream)>>>(policy_logps, lengths, n_samples, lambda, loss, coef,
+  psa::launch_behind(true, psa::orpo_loss_kernel, dim3(1), 256, 0, cudaStream_t(stream), policy_logps, lengths, n_samples, lambda, loss, coef,
                                                             device_status);
   return psa::check_last_cuda_error("orpo_loss launch");
 }

@@ -33,6 +33,7 @@
 
 #include "psa_device.cuh"
 #include "psa_internal.h"
+#include "psa_launch.cuh"
 #include "psa_tensormap.h"
 
 namespace psa {
@@ -167,6 +168,7 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  behind_go();
 
   // Iteration it (of this CTA) -> (query head of the group, entry of the list).
   auto head_of = [&](int it) { return hk * g + (kSplit ? it0 + it : it) / n_list; };
@@ -299,6 +301,7 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     // Thread = one key row (TMEM lane) and one half of the 128 query columns: warps 4..7 take
     // columns [0,64), warps 8..11 columns [64,128).
     setmaxnreg_inc<144>();
+    behind_wait();   // delta
     constexpr int DH = D / 2;                           // dV / dK columns per worker in the epilogue
     const int quarter = warp & 3;
     const int half = (warp - 4) >> 2;
@@ -685,6 +688,7 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   } else {
     // ------------------------------------------------------------ dQ drain: warps 12..15, one query row per thread
     setmaxnreg_inc<152>();
+    behind_wait();   // the accumulator is cleared
     const int quarter = warp & 3;
     const int r = quarter * 32 + lane;
     const uint32_t lane_base = uint32_t(quarter * 32) << 16;
@@ -756,6 +760,8 @@ psa_bwd_delta_kernel(const __nv_bfloat16* __restrict__ d_o, const __nv_bfloat16*
                      float* __restrict__ delta, float* __restrict__ dq_accum, int64_t row0,
                      int64_t row1 /* of T*Hq */, int32_t T, int32_t Hq, int32_t* status) {
   constexpr int kLanes = D / 8;  // threads per (t, h) row
+  behind_wait();
+  behind_go();
   const int64_t gid = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   const int64_t row = row0 + gid / kLanes;
   const int part = int(gid % kLanes);
@@ -835,6 +841,8 @@ psa_bwd_delta_few_keys_kernel(const FewKeyRow* __restrict__ rows, const __nv_bfl
 __global__ void __launch_bounds__(256)
 psa_bwd_convert_kernel(const float4* __restrict__ acc, uint2* __restrict__ dq, int64_t n_vec4) {
   const int64_t base = (int64_t(blockIdx.x) * blockDim.x) * 4 + threadIdx.x;
+  behind_wait();
+  behind_go();
   float4 a[4];
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
@@ -879,11 +887,19 @@ psa_status_t launch_bwd_t(const psa_plan_t* plan, const PlanPart& part, const vo
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kRequest) != cudaSuccess)
     return PSA_ERR_CUDA;
 
+  // In launches of one wave each kernel starts behind the one before it: 276 tokens, 4 heads of 64, backward 15.0 -> 13.5
+  // us; 1500 tokens, 8/2 heads, 34.2 -> 33.4.  Longer ones lose: a CTA that is early takes an SM from the passes over dq
+  // (6860 tokens, 32/8 heads of 128: 204 -> 212).  The two passes over dq only where every block
+  // finds an SM of its own: those that start early fill the few idle SMs, and stay there (4004 tokens, 4 heads of 64, a
+  // conversion of 250 blocks beside 128 CTAs: backward 62.5 -> 65.1 us).
+  const int one_wave = part.n_ctas * split;
+  const bool behind = one_wave <= plan->n_sm;
   const int64_t row0 = int64_t(part.row0) * plan->Hq, row1 = int64_t(part.row1) * plan->Hq, n_rows = row1 - row0;
   {
     ProfileScope prof(3, stream);
     const int64_t threads = n_rows * (D / 8);
-    psa_bwd_delta_kernel<D><<<unsigned((threads + 255) / 256), 256, 0, stream>>>(
+    const int64_t blocks = (threads + 255) / 256;
+    launch_behind(behind && blocks <= plan->n_sm, psa_bwd_delta_kernel<D>, dim3(unsigned(blocks)), 256, 0, stream,
         static_cast<const __nv_bfloat16*>(d_o), static_cast<const __nv_bfloat16*>(o), delta, dq_accum, row0, row1,
         plan->T, plan->Hq, device_status);
   }
@@ -914,12 +930,14 @@ psa_status_t launch_bwd_t(const psa_plan_t* plan, const PlanPart& part, const vo
   cfg.blockDim = dim3(kBwdThreads);
   cfg.dynamicSmemBytes = L::kRequest;
   cfg.stream = stream;
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = unsigned(split);
-  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = split > 1 ? 1 : 0;
+  cudaLaunchAttribute attr[2] = {};
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = unsigned(split);
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = split > 1 ? attr : attr + 1;
+  cfg.numAttrs = (split > 1 ? 1 : 0) + (behind ? 1 : 0);
   {
     ProfileScope prof(1, stream);
     cudaLaunchKernelEx(&cfg, kernel, tm_q, tm_k, tm_v, tm_do, tm_dq, tm_dk, tm_dv, prm);
@@ -927,7 +945,8 @@ psa_status_t launch_bwd_t(const psa_plan_t* plan, const PlanPart& part, const vo
   if (!f32_out) {
     ProfileScope prof(4, stream);
     const int64_t n_vec4 = n_rows * D / 4;
-    psa_bwd_convert_kernel<<<unsigned((n_vec4 + 1023) / 1024), 256, 0, stream>>>(
+    const int64_t blocks = (n_vec4 + 1023) / 1024;
+    launch_behind(one_wave + blocks <= plan->n_sm, psa_bwd_convert_kernel, dim3(unsigned(blocks)), 256, 0, stream,
         reinterpret_cast<const float4*>(dq_accum) + row0 * D / 4, static_cast<uint2*>(dq) + row0 * D / 4, n_vec4);
   }
   return check_last_cuda_error("psa_bwd launch");

@@ -27,6 +27,7 @@
 
 #include "psa_device.cuh"
 #include "psa_internal.h"
+#include "psa_launch.cuh"
 #include "psa_tensormap.h"
 
 namespace psa {
@@ -120,6 +121,8 @@ psa_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     return ItemView{im.rec, im.h, im.hk, im.n_it, prm.entries + im.rec.list_off, s_ent_all + item * L::kEntCap};
   };
 
+  behind_wait();
+  behind_go();
   if (threadIdx.x == 32 && n_items == 2) {   // the second item's record, while thread 0 requests the first tiles
     const int h1 = idx1 % prm.Hq;
     const TileRec r1 = prm.tiles[idx1 / prm.Hq];
@@ -685,7 +688,10 @@ psa_status_t launch_fwd_t(const psa_plan_t* plan, const PlanPart& part, const vo
   const unsigned grid = unsigned(prm.n_items + prm.items_per_cta - 1) / unsigned(prm.items_per_cta);
   {
     ProfileScope prof(0, stream);
-    psa_fwd_kernel<D><<<grid, kFwdThreads, L::kRequest, stream>>>(tm_q, tm_k, tm_v, tm_o, prm);
+    // A launch of one wave starts behind the kernel before it (276 tokens, 4 heads of 64: 8.4 -> 7.8 us; 1142 tokens, 8/2
+    // heads of 128: 18.4 -> 18.0); a longer one has other things to wait for.
+    launch_behind(grid <= 2u * unsigned(plan->n_sm), psa_fwd_kernel<D>, dim3(grid), kFwdThreads, L::kRequest, stream, tm_q,
+                  tm_k, tm_v, tm_o, prm);
   }
   return check_last_cuda_error("psa_fwd launch");
 }

@@ -51,6 +51,7 @@ struct PlanPart {
 
 struct psa_plan {
   int32_t n_samples = 0, T = 0, Hq = 0, Hkv = 0, d = 0;
+  int32_t n_sm = 148;             // of the device that the plan was made on
   float scale = 0.f;
   int64_t useful_pairs = 0, live_tiles = 0, partial_tiles = 0;
   size_t bwd_workspace_bytes = 0;

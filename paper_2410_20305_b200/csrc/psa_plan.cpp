@@ -274,6 +274,7 @@ extern "C" psa_status_t psa_plan(const int32_t* cu_seqlens, const int32_t* prefi
           cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
         n_sm = v;
     }
+    p->n_sm = n_sm;
     // Key tiles of every sample, longest list first.
     std::vector<std::vector<int32_t>> tiles_of(n_samples);
     for (size_t t = 0; t < p->kv_tiles.size(); ++t) {

@@ -1,0 +1,82 @@
+"""Launches that start behind one another (small packs, the loss chain) see what the kernels before them have written."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2410_20305_b200 import binding as B
+from paper_2410_20305_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+def _dev(a):
+    return torch.as_tensor(np.asarray(a, dtype=np.int32)).cuda()
+
+
+def _inputs(seed, n, longest, heads, dtype, vocab):
+    pack = wl.random_pack(seed, n, longest, *heads)
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    q, k, v, d_o = (t.cuda() for t in wl.attention_inputs(pack, seed))
+    T = pack.total_tokens
+    logits = torch.randn((T, (vocab + 7) // 8 * 8), generator=gen, device="cuda").to(dtype)[:, :vocab]
+    tok = np.random.default_rng(seed).integers(0, vocab, T).astype(np.int32)
+    labels = B.psa_logp_labels(tok, pack.cu_seqlens, pack.prefix_len, pack.chosen_len, pack.rejected_len)
+    lengths = np.maximum(np.bincount(labels[1][labels[1] >= 0], minlength=2 * pack.n_samples), 1)
+    return pack, (q, k, v, d_o), logits, [_dev(a) for a in labels], _dev(lengths)
+
+
+def _step(pack, qkv, logits, labels, lengths, f32):
+    """Every call of a training step; all outputs."""
+    q, k, v, d_o = qkv
+    plan = B.psa_plan(pack.cu_seqlens, pack.prefix_len, pack.chosen_len, pack.rejected_len, pack.n_q_heads, pack.n_kv_heads,
+                      pack.head_dim)
+    ws = torch.empty(plan.bwd_workspace_bytes, dtype=torch.uint8, device="cuda")
+    pos = _dev(B.psa_position_ids(pack.cu_seqlens, pack.prefix_len, pack.chosen_len, pack.rejected_len))
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    qr = B.psa_rope(q, pos, 10000.0, out=torch.empty_like(q))
+    o, lse = B.psa_fwd(plan, qr, k, v, o=torch.empty_like(q), lse=None, status=status)
+    targets, segments, *forks = labels
+    lp = B.dpo_logp(logits, targets, segments, 2 * pack.n_samples, *forks, status=status)
+    outs = [qr, o, lse, lp]
+    for loss, coef in (B.dpo_loss(lp, lp * 1.01, 0.1), B.simpo_loss(lp, lengths, 2.0, 0.5), B.orpo_loss(lp, lengths, 0.1)):
+        d = torch.empty_strided(logits.shape, logits.stride(), dtype=logits.dtype, device="cuda")
+        outs += [loss, coef, B.dpo_logp_bwd(logits, targets, segments, coef, *forks, dlogits=d, status=status)]
+    backward = B.psa_bwd_f32 if f32 else B.psa_bwd
+    g = [torch.empty(t.shape, dtype=torch.float32 if f32 else t.dtype, device="cuda") for t in (q, k, v)]
+    outs += backward(plan, d_o, qr, k, v, o, lse, *g, workspace=ws, status=status)
+    return outs, status
+
+
+def _same(got, want):
+    for i, (a, b) in enumerate(zip(got, want)):
+        if i == len(want) - 3 or i >= 3 and i < 13:
+            # dq: fp32 adds in any order, at most one rounding of the output apart.  The log-probs' fp64 sums come in any
+            # order too, one fp32 rounding apart, and what follows from them.
+            assert torch.allclose(a.float(), b.float(), rtol=2.0 ** -7, atol=1e-5)
+        else:
+            assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("seed,n,longest,heads", [(1, 1, 130, (4, 4, 64)), (2, 2, 400, (8, 2, 128)), (4, 3, 90, (4, 2, 64))])
+def test_launches_behind_one_another_see_what_came_before(seed, n, longest, heads):
+    """Inputs and labels are rewritten on the stream right before every step, and the same buffers are used again."""
+    pack, qkv, logits, labels, lengths = _inputs(seed, n, longest, heads, torch.bfloat16, 504)
+    variants = [([t * s for t in qkv], logits * s) for s in (1.0, 0.5, -1.0)]
+    want = []
+    for x, y in variants:
+        torch.cuda.synchronize()
+        outs, _ = _step(pack, x, y, labels, lengths, False)
+        torch.cuda.synchronize()
+        want.append([t.clone() for t in outs])
+    live_x, live_y = [torch.empty_like(t) for t in qkv], torch.empty_strided(logits.shape, logits.stride(), dtype=logits.dtype,
+                                                                          device="cuda")
+    torch.cuda.synchronize()
+    for turn in range(30):
+        x, y = variants[turn % 3]
+        for a, b in zip(live_x, x):
+            a.copy_(b)
+        live_y.copy_(y)
+        outs, status = _step(pack, live_x, live_y, labels, lengths, False)
+        kept = [t.clone() for t in outs]
+        _same(kept, want[turn % 3])
+        assert int(status.item()) == 0
