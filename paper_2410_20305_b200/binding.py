@@ -93,7 +93,37 @@ def load_library():
         elif name != "psa_status_string":
             getattr(lib, name).restype = C.c_int
     _lib = lib
+    _load_native(lib, _build)
     return lib
+
+
+# The compiled route of the calls below (csrc/psa_native.cpp), or None.  It takes a call on the current stream whose
+# arguments are as they have to be, and returns None for any other, which then goes on here.
+_native = None
+_NATIVE_ENTRIES = ("psa_fwd", "psa_bwd", "psa_bwd_f32", "dpo_logp_f64sum", "dpo_logp_bwd", "dpo_loss", "simpo_loss",
+                   "orpo_loss", "psa_rope", "psa_plan", "psa_plan_stats", "psa_plan_destroy")
+
+
+def _load_native(lib, build):
+    global _native
+    try:
+        import torch  # noqa: F401  (its libraries have to be there before the extension's)
+        from importlib.machinery import ExtensionFileLoader
+        from importlib.util import module_from_spec, spec_from_loader
+        loader = ExtensionFileLoader("psa_native", build.build_native())
+        module = module_from_spec(spec_from_loader("psa_native", loader))
+        loader.exec_module(module)
+        if module.init(tuple(C.cast(getattr(lib, name), C.c_void_p).value for name in _NATIVE_ENTRIES)):
+            _native = module
+    except Exception:   # without a compiler or torch's headers: every call goes through ctypes
+        _native = None
+
+
+def _fast(stream):
+    """The compiled route, where the call is on the current stream and `load_library` is the one above."""
+    if stream is None and load_library is _load_library:
+        return _native if _lib is not None else (load_library() and _native)
+    return None
 
 
 def _check(fn, code):
@@ -105,6 +135,9 @@ def _i32(a):
     if type(a) is np.ndarray and a.dtype == np.int32 and a.flags.c_contiguous:
         return a
     return np.ascontiguousarray(np.asarray(a, dtype=np.int32))
+
+
+_load_library = load_library   # (`load_library` itself may be replaced, for instance to write calls down)
 
 
 # Pointers and streams are handed over as plain integers (every such argument is declared c_void_p).
@@ -175,12 +208,21 @@ def _want_attention(plan, bf16, f32=(), lse=None, cuda=True):
             _want(lse, "lse", (plan.n_q_heads, T), torch.float32, cuda, placement)
 
 
+def _cuda_ready():
+    import torch
+    return torch.cuda.is_initialized()
+
+
 class Plan:
     """Owner of a psa_plan_t*.  One plan serves every layer of a step."""
 
-    def __init__(self, handle, n_q_heads, n_kv_heads, head_dim):
+    def __init__(self, handle, n_q_heads, n_kv_heads, head_dim, stats=None):
         self._h = handle
         self.n_q_heads, self.n_kv_heads, self.head_dim = n_q_heads, n_kv_heads, head_dim
+        if stats is not None:
+            self.total_tokens, self.useful_pairs, self.live_tiles, self.partial_tiles, self.bwd_workspace_bytes = stats
+            self._key = (handle.value, self.total_tokens, n_q_heads, n_kv_heads, head_dim, self.bwd_workspace_bytes)
+            return
         lib = load_library()
         T, U, live, part = C.c_int64(), C.c_int64(), C.c_int64(), C.c_int64()
         ws = C.c_size_t()
@@ -188,6 +230,7 @@ class Plan:
                                                     C.byref(ws)))
         self.total_tokens, self.useful_pairs = T.value, U.value
         self.live_tiles, self.partial_tiles, self.bwd_workspace_bytes = live.value, part.value, ws.value
+        self._key = (handle.value, T.value, n_q_heads, n_kv_heads, head_dim, ws.value)
 
     def upload(self, stream=None):
         _check("psa_plan_upload", load_library().psa_plan_upload(self._h, _stream(stream)))
@@ -211,8 +254,12 @@ class Plan:
 
     def close(self):
         if self._h:
-            h, self._h = self._h, None
-            load_library().psa_plan_destroy(h)
+            h, self._h, self._key = self._h, None, None
+            fast = _fast(None)
+            if fast:
+                fast.destroy(h.value)
+            else:
+                load_library().psa_plan_destroy(h)
 
     def __del__(self):
         try:
@@ -223,6 +270,13 @@ class Plan:
 
 def psa_plan(cu_seqlens, prefix_len, chosen_len, rejected_len, n_q_heads, n_kv_heads, head_dim,
              softmax_scale=0.0, host_only=False, stream=None) -> Plan:
+    fast = None if host_only else _fast(stream)
+    if fast and _cuda_ready():
+        made = fast.plan(cu_seqlens, prefix_len, chosen_len, rejected_len, n_q_heads, n_kv_heads, head_dim, float(softmax_scale))
+        if type(made) is tuple:
+            return Plan(C.c_void_p(made[0]), n_q_heads, n_kv_heads, head_dim, made[1:])
+        if made is not None:
+            _check("psa_plan", made)
     lib = load_library()
     cu, P, Cc, R = _i32(cu_seqlens), _i32(prefix_len), _i32(chosen_len), _i32(rejected_len)
     n = len(P)
@@ -244,6 +298,12 @@ def psa_fwd(plan: Plan, q, k, v, o=None, lse=None, status=None, stream=None):
         o = torch.empty_like(q)
     if lse is None:
         lse = torch.empty((plan.n_q_heads, T), dtype=torch.float32, device=q.device)
+    fast = _fast(stream)
+    if fast:
+        code = fast.fwd(plan._key, q, k, v, o, lse, status)
+        if code is not None:
+            _check("psa_fwd", code)
+            return o, lse
     _want_attention(plan, [("q", q, "q"), ("k", k, "kv"), ("v", v, "kv"), ("o", o, "q")], lse=lse)
     _check("psa_fwd", load_library().psa_fwd(plan._h, _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse), _ptr(status),
                                              _stream(stream)))
@@ -259,6 +319,12 @@ def psa_bwd(plan: Plan, d_o, q, k, v, o, lse, dq=None, dk=None, dv=None, workspa
         dk = torch.empty_like(k)
     if dv is None:
         dv = torch.empty_like(v)
+    fast = _fast(stream) if workspace is not None else None
+    if fast:
+        code = fast.bwd(False, plan._key, d_o, q, k, v, o, lse, dq, dk, dv, workspace, status)
+        if code is not None:
+            _check("psa_bwd", code)
+            return dq, dk, dv
     _want_attention(plan, [("d_o", d_o, "q"), ("q", q, "q"), ("k", k, "kv"), ("v", v, "kv"), ("o", o, "q"),
                            ("dq", dq, "q"), ("dk", dk, "kv"), ("dv", dv, "kv")], lse=lse)
     if workspace is None:
@@ -279,6 +345,12 @@ def psa_bwd_f32(plan: Plan, d_o, q, k, v, o, lse, dq=None, dk=None, dv=None, wor
     dq = f32(q) if dq is None else dq
     dk = f32(k) if dk is None else dk
     dv = f32(v) if dv is None else dv
+    fast = _fast(stream) if workspace is not None else None
+    if fast:
+        code = fast.bwd(True, plan._key, d_o, q, k, v, o, lse, dq, dk, dv, workspace, status)
+        if code is not None:
+            _check("psa_bwd_f32", code)
+            return dq, dk, dv
     _want_attention(plan, [("d_o", d_o, "q"), ("q", q, "q"), ("k", k, "kv"), ("v", v, "kv"), ("o", o, "q")],
                     f32=[("dq", dq, "q"), ("dk", dk, "kv"), ("dv", dv, "kv")], lse=lse)
     if workspace is None:
@@ -317,6 +389,13 @@ def dpo_logp(logits, targets, segment_ids, n_segments, fork_rows=None, fork_targ
     int32 [n_rows], optional fork arrays int32 [n_forks] -> out fp32 [n_segments].
     `scratch` (optional): a CUDA buffer of at least 8 * (n_segments + 1) bytes for the fp64 sums,
     in use until the call's work on the stream has ended."""
+    fast = _fast(stream) if out is None and scratch is None else None
+    if fast:
+        got = fast.logp(logits, targets, segment_ids, n_segments, fork_rows, fork_targets, fork_segments, status)
+        if type(got) is int:
+            _check("dpo_logp", got)
+        elif got is not None:
+            return got
     import torch
     assert logits.is_cuda and logits.dim() == 2 and logits.stride(1) == 1
     dt = {torch.float32: PSA_DTYPE_F32, torch.bfloat16: PSA_DTYPE_BF16}[logits.dtype]
@@ -395,6 +474,13 @@ def psa_step_host(plan: Plan, h_q, h_k, h_v, h_do, h_o, h_lse, h_dq, h_dk, h_dv,
 def dpo_loss(policy_logps, ref_logps, beta, stream=None):
     """policy_logps, ref_logps fp32 CUDA [2n] (2s chosen, 2s+1 rejected) -> (loss fp32 [1], coef fp32 [2n])
     with coef = d loss / d policy_logps; loss = mean_s -log sigmoid(beta * margin_s)."""
+    fast = _fast(stream)
+    if fast:
+        got = fast.loss(0, policy_logps, ref_logps, float(beta), 0.0, None)
+        if type(got) is tuple:
+            return got
+        if got is not None:
+            _check("dpo_loss", got)
     import torch
     assert policy_logps.is_cuda and policy_logps.dtype == torch.float32 and policy_logps.is_contiguous()
     assert ref_logps.shape == policy_logps.shape and ref_logps.dtype == torch.float32 and ref_logps.is_contiguous()
@@ -409,6 +495,13 @@ def dpo_loss(policy_logps, ref_logps, beta, stream=None):
 def simpo_loss(policy_logps, lengths, beta, gamma, status=None, stream=None):
     """policy_logps fp32 CUDA [2n], lengths int32 CUDA [2n] (scored tokens per response) ->
     (loss fp32 [1], coef fp32 [2n]); loss = mean_s -log sigmoid(beta * (lp_c/len_c - lp_r/len_r) - gamma)."""
+    fast = _fast(stream)
+    if fast:
+        got = fast.loss(1, policy_logps, lengths, float(beta), float(gamma), status)
+        if type(got) is tuple:
+            return got
+        if got is not None:
+            _check("simpo_loss", got)
     import torch
     assert policy_logps.is_cuda and policy_logps.dtype == torch.float32 and policy_logps.is_contiguous()
     assert lengths.is_cuda and lengths.dtype == torch.int32 and lengths.shape == policy_logps.shape
@@ -424,6 +517,13 @@ def simpo_loss(policy_logps, lengths, beta, gamma, status=None, stream=None):
 def orpo_loss(policy_logps, lengths, lam, status=None, stream=None):
     """policy_logps fp32 CUDA [2n], lengths int32 CUDA [2n] -> (loss fp32 [1], coef fp32 [2n]);
     loss = mean_s  -lp_c/len_c + lam * -log sigmoid(log odds ratio of the mean-token likelihoods)."""
+    fast = _fast(stream)
+    if fast:
+        got = fast.loss(2, policy_logps, lengths, float(lam), 0.0, status)
+        if type(got) is tuple:
+            return got
+        if got is not None:
+            _check("orpo_loss", got)
     import torch
     assert policy_logps.is_cuda and policy_logps.dtype == torch.float32 and policy_logps.is_contiguous()
     assert lengths.is_cuda and lengths.dtype == torch.int32 and lengths.shape == policy_logps.shape
@@ -439,6 +539,12 @@ def dpo_logp_bwd(logits, targets, segment_ids, coef, fork_rows=None, fork_target
                  dlogits=None, status=None, stream=None):
     """Gradient of sum_g coef[g] * dpo_logp(...)[g] with respect to the logits; same dtype and
     row stride as `logits`."""
+    fast = _fast(stream) if dlogits is not None else None
+    if fast:
+        code = fast.logp_bwd(logits, targets, segment_ids, coef, fork_rows, fork_targets, fork_segments, dlogits, status)
+        if code is not None:
+            _check("dpo_logp_bwd", code)
+            return dlogits
     import torch
     assert logits.is_cuda and logits.dim() == 2 and logits.stride(1) == 1
     dt = {torch.float32: PSA_DTYPE_F32, torch.bfloat16: PSA_DTYPE_BF16}[logits.dtype]
@@ -525,6 +631,12 @@ def psa_position_ids(cu_seqlens, prefix_len, chosen_len, rejected_len):
 def psa_rope(x, position_ids, rope_theta=10000.0, out=None, stream=None):
     """Rotary embedding (rotate-half convention) of x [T, H, d] bf16 CUDA with int32 CUDA position ids [T]."""
     import torch
+    fast = _fast(stream) if out is not None else None
+    if fast:
+        code = fast.rope(x, position_ids, float(rope_theta), out)
+        if code is not None:
+            _check("psa_rope", code)
+            return out
     assert x.is_cuda and x.dtype == torch.bfloat16 and x.is_contiguous() and x.dim() == 3
     assert position_ids.is_cuda and position_ids.dtype == torch.int32 and position_ids.numel() == x.shape[0]
     if out is None:

@@ -10,6 +10,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libpsa.so")
 LIB_DEBUG = os.path.join(HERE, "libpsa_debug.so")   # the same sources with -DPSA_DEBUG_BOUNDS (checked global indices)
+NATIVE = os.path.join(HERE, "psa_native.so")
 SOURCES = ["psa_plan.cpp", "psa_host_helpers.cpp", "psa_api.cu", "psa_fwd.cu", "psa_bwd.cu", "psa_bwd_static.cu", "psa_selftest.cu",
            "dpo_logp.cu", "dpo_loss.cu", "psa_rope.cu"]
 
@@ -18,7 +19,7 @@ def _stale(lib=LIB) -> bool:
     if not os.path.exists(lib):
         return True
     t = os.path.getmtime(lib)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "psa.h")]
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != "psa_native.cpp"] + [os.path.join(ROOT, "include", "psa.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
@@ -44,6 +45,32 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
     return lib
 
 
+def build_native(force: bool = False) -> str:
+    """Builds psa_native.so, the compiled route of the binding's calls (csrc/psa_native.cpp), against the torch that runs."""
+    source = os.path.join(CSRC, "psa_native.cpp")
+    deps = [source, os.path.join(ROOT, "include", "psa.h")]
+    if not force and os.path.exists(NATIVE) and all(os.path.getmtime(d) <= os.path.getmtime(NATIVE) for d in deps):
+        return NATIVE
+    import sysconfig
+    import torch
+    home = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    include = [os.path.join(ROOT, "include"), os.path.join(home, "include"),
+               os.path.join(home, "include", "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"],
+               os.path.join(cuda, "include")]
+    # into place at once: another process may be about to load it
+    out = "%s.%d.tmp" % (NATIVE, os.getpid())
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI]
+    cmd += [a for d in include for a in ("-I", d)] + ["-o", out, source, "-L", os.path.join(home, "lib")]
+    cmd += ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("g++ failed building psa_native.so: " + res.stderr[-2000:])
+    os.replace(out, NATIVE)
+    return NATIVE
+
+
 if __name__ == "__main__":
     print(build(force=True, verbose=True))
     print(build(force=True, debug=True))
+    print(build_native(force=True))

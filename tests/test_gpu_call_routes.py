@@ -1,10 +1,13 @@
-"""Launches that start behind one another (small packs, the loss chain) see what the kernels before them have written."""
+"""The binding's compiled route and its ctypes route are one: same results, same refusals.  And launches that start behind
+one another (small packs, the loss chain) see what the kernels before them have written."""
 import numpy as np
 import pytest
 import torch
 
 from paper_2410_20305_b200 import binding as B
 from paper_2410_20305_b200 import workloads as wl
+
+from gpu_util import device_plan
 
 pytestmark = pytest.mark.gpu
 
@@ -55,6 +58,56 @@ def _same(got, want):
             assert torch.allclose(a.float(), b.float(), rtol=2.0 ** -7, atol=1e-5)
         else:
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("heads,f32,dtype", [((4, 2, 64), False, torch.bfloat16), ((8, 2, 128), True, torch.float32)])
+def test_both_routes_give_the_same_step(monkeypatch, heads, f32, dtype):
+    args = _inputs(3, 3, 200, heads, dtype, 1003)
+    assert B.load_library() and B._native is not None
+    got, status = _step(*args, f32)
+    monkeypatch.setattr(B, "_native", None)
+    want, other = _step(*args, f32)
+    assert int(status.item()) == int(other.item()) == 0
+    _same(got, want)
+
+
+def test_both_routes_refuse_the_same_calls(monkeypatch):
+    pack, (q, k, v, d_o), logits, labels, lengths = _inputs(5, 2, 150, (4, 2, 64), torch.bfloat16, 256)
+    plan = device_plan(pack)
+    o, lse = B.psa_fwd(plan, q, k, v)
+    ws = torch.empty(plan.bwd_workspace_bytes, dtype=torch.uint8, device="cuda")
+    g = [torch.empty_like(t) for t in (q, k, v)]
+    lp = torch.zeros(2 * pack.n_samples, device="cuda")
+    flat = q.transpose(0, 1).contiguous().transpose(0, 1)
+    calls = [
+        lambda: B.psa_fwd(plan, q[:-1], k, v), lambda: B.psa_fwd(plan, q.float(), k, v), lambda: B.psa_fwd(plan, q, k.cpu(), v),
+        lambda: B.psa_fwd(plan, flat, k, v), lambda: B.psa_fwd(plan, q, k, v, lse=lse[:, :-1]),
+        lambda: B.psa_bwd(plan, d_o, q, k, v, o, lse, *g, workspace=ws[:-1]),
+        lambda: B.psa_bwd(plan, d_o, q, k, v, o, lse, *g, workspace=ws.cpu()),
+        lambda: B.psa_bwd_f32(plan, d_o, q, k, v, o, lse, *g, workspace=ws),
+        lambda: B.psa_plan(pack.cu_seqlens[:-1], pack.prefix_len, pack.chosen_len, pack.rejected_len, 4, 2, 64),
+        lambda: B.psa_plan(pack.cu_seqlens + 1, pack.prefix_len, pack.chosen_len, pack.rejected_len, 4, 2, 64),
+        lambda: B.psa_plan(pack.cu_seqlens, pack.prefix_len, pack.chosen_len, pack.rejected_len, 4, 3, 64),
+        lambda: B.dpo_logp(logits, labels[0][:-1], labels[1], 4), lambda: B.dpo_logp(logits.cpu(), labels[0], labels[1], 4),
+        lambda: B.dpo_logp(logits, labels[0].long(), labels[1], 4), lambda: B.dpo_logp(logits, labels[0], labels[1], -1),
+        lambda: B.dpo_logp_bwd(logits, labels[0], labels[1], lp.double(), dlogits=torch.empty_like(logits)),
+        lambda: B.dpo_logp_bwd(logits, labels[0], labels[1], lp, dlogits=torch.empty_like(logits).float()),
+        lambda: B.dpo_loss(lp, lp[:-1], 0.1), lambda: B.simpo_loss(lp, lp, 0.1, 0.2), lambda: B.orpo_loss(lp.double(), lengths, 0.1),
+        lambda: B.psa_rope(q.float(), labels[0], out=q), lambda: B.psa_rope(q, labels[0][:-1], out=q),
+    ]
+    for route in (B._native, None):
+        monkeypatch.setattr(B, "_native", route)
+        said = []
+        for i, call in enumerate(calls):
+            with pytest.raises(Exception) as e:
+                call()
+            said.append((i, type(e.value), str(e.value)))
+        if route is not None:
+            first = said
+    assert said == first
+    plan.close()
+    with pytest.raises(B.PsaError):
+        B.psa_fwd(plan, q, k, v, o=o, lse=lse)
 
 
 @pytest.mark.parametrize("seed,n,longest,heads", [(1, 1, 130, (4, 4, 64)), (2, 2, 400, (8, 2, 128)), (4, 3, 90, (4, 2, 64))])
