@@ -88,10 +88,15 @@ void items_per_cta(const psa_plan_t* p, int n_sm, PlanPart* part) {
 //
 // Order: every CTA adds its dQ contributions into the fp32 accumulator rows of its sample and query-head group, so CTAs
 // that share those rows are launched together: the rows then stay in L2 while they are being updated.  Samples with
-// the most work first, then kv head, then the sample's key tiles, longest list first.  That can leave a ragged tail
-// (its makespan over 148 SMs is 8 % above the mean on the Llama-3-8B-shaped pack).  Alternative: hand out the last 30 %
-// of the work longest first.  That evens out the finish but gives up the L2 locality of the tail, so it is taken only
-// when a list-scheduling simulation says it shortens the makespan by more than 5 %.
+// the most work first, then kv head, then the sample's key tiles, longest list first.  That can leave a ragged tail, so
+// the end of the order is handed out longest first: the last wave and a bit (115 % of one pair per SM), or, where the
+// whole accumulator stays in L2 anyway, 30 %, 50 % or all of it, whichever a list-scheduling simulation finds shortest.
+// It has to be 1.5 % shorter than the grouped order.  us of the whole backward with the last 0 / 5 / 10 / 20 / 30 / 100 %
+// longest first (before: 30 %, where that was 5 % shorter in the simulation):
+//   31041 tokens, 32/8 heads of 128 (13 waves)  2398 / 2352 / 2366 / 2458 / 2512 / 2598
+//   19431, 32/8 of 128 (8)    1039 / 1031 / 1015 / 1028 / 1046 / 1107     16215, 32/8 of 128 (7)  892 / 893 / 871 / 850 / 864 / 930
+//   7727, 32/8 of 128 (3.7)   226 / 224 / 223 / 218 / 211 / 227           accumulators of 19 to 42 MB:
+//   4952, 8/8 of 128 (2.2)    109 / 110 / 106 / 101 / 96 / 91             5465, 32/8 of 64 (2.4)  223 / 222 / 217 / 204 / 191 / 166
 void order_backward(psa_plan_t* p, const std::vector<std::vector<int32_t>>& tiles_of, int s0, int s1, int n_sm,
                     PlanPart* part) {
   typedef std::vector<std::pair<int32_t, int32_t>> Order;   // (key tile record, kv head)
@@ -101,12 +106,12 @@ void order_backward(psa_plan_t* p, const std::vector<std::vector<int32_t>>& tile
   std::vector<int> order(s1 - s0);
   std::iota(order.begin(), order.end(), s0);
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return work[a - s0] > work[b - s0]; });
-  Order ctas;
+  Order grouped;
   int64_t total_work = 0;
   for (int s : order)
     for (int hk = 0; hk < p->Hkv; ++hk)
       for (int32_t t : tiles_of[s]) {
-        ctas.emplace_back(t, hk);
+        grouped.emplace_back(t, hk);
         total_work += p->kv_tiles[t].list_cnt;
       }
   // Makespan of an order on `slots` slots, a pair with a list of n taking cost(n).
@@ -132,16 +137,34 @@ void order_backward(psa_plan_t* p, const std::vector<std::vector<int32_t>>& tile
     }
     return end;
   };
-  if (part == &p->whole) {
-    Order hybrid = ctas;
+  const int64_t iter_ns = p->d == 128 ? 2050 : 1600, fixed_ns = p->d == 128 ? 8000 : 7000, combine_ns = 3000;
+  const int64_t group = p->Hq / p->Hkv;
+  auto alone = [&](int32_t n) { return n * group * iter_ns + fixed_ns; };
+  // The pairs with the last `permille` of the work longest first.
+  auto tail_sorted = [&](int64_t permille) {
+    Order o = grouped;
     int64_t acc = 0;
     size_t at = 0;
-    while (at < hybrid.size() && acc * 10 < total_work * 7) acc += p->kv_tiles[hybrid[at++].first].list_cnt;
-    std::stable_sort(hybrid.begin() + at, hybrid.end(), [&](const auto& a, const auto& b) {
+    while (at < o.size() && acc * 1000 < total_work * (1000 - permille)) acc += p->kv_tiles[o[at++].first].list_cnt;
+    std::stable_sort(o.begin() + at, o.end(), [&](const auto& a, const auto& b) {
       return p->kv_tiles[a.first].list_cnt > p->kv_tiles[b.first].list_cnt;
     });
-    auto length = [](int32_t n) { return int64_t(n); };
-    if (makespan(ctas, n_sm, length) * 100 > makespan(hybrid, n_sm, length) * 105) ctas.swap(hybrid);
+    return o;
+  };
+  Order ctas = grouped;
+  int64_t best = makespan(ctas, n_sm, alone);
+  if (part == &p->whole && grouped.size() > size_t(n_sm)) {
+    const bool in_l2 = int64_t(p->T) * p->Hq * p->d * 4 <= (int64_t(64) << 20);
+    const int64_t wave = std::min<int64_t>(1000, 1150 * int64_t(n_sm) / int64_t(grouped.size()));
+    int64_t shortest = best * 985 / 1000;
+    for (int64_t permille : {wave, int64_t(300), int64_t(500), int64_t(1000)}) {
+      if (permille != wave && !in_l2) break;
+      Order o = tail_sorted(permille);
+      const int64_t t = makespan(o, n_sm, alone);
+      if (t >= shortest) continue;
+      shortest = best = t;
+      ctas.swap(o);
+    }
   }
   // CTAs per pair: where the pairs are few, the longest of them lasts longer than the rest of the chip is busy.  Sharing
   // a pair costs each of its CTAs the fixed part of a CTA and the reduction over the cluster, so it only pays below two
@@ -154,12 +177,12 @@ void order_backward(psa_plan_t* p, const std::vector<std::vector<int32_t>>& tile
   if (part != &p->whole) {
     part->bwd_split = p->whole.bwd_split;   // dk and dv are summed in the same order, and come out the same, as for the whole
   } else if (ctas.size() <= 2 * size_t(n_sm)) {
-    const int64_t iter_ns = p->d == 128 ? 2050 : 1600, fixed_ns = p->d == 128 ? 8000 : 7000, combine_ns = 3000;
-    const int64_t group = p->Hq / p->Hkv;
-    int64_t best = makespan(ctas, n_sm, [&](int32_t n) { return n * group * iter_ns + fixed_ns; });
+    // Pairs that share their iterations are few, and handed out longest first as a whole (2008 tokens, 32/8 heads of 128,
+    // 145 -> 103 us; 2436 tokens, 32/8 of 64, 151 -> 110).
+    Order sorted = tail_sorted(1000);
     for (int split : {2, 4, 8}) {
       const size_t slots = split == 2 ? n_sm / 2 : (split == 4 ? n_sm * 33 / 148 : n_sm * 15 / 148);
-      const int64_t t = makespan(ctas, std::max<size_t>(slots, 1), [&](int32_t n) {
+      const int64_t t = makespan(sorted, std::max<size_t>(slots, 1), [&](int32_t n) {
         return (n * group + split - 1) / split * iter_ns + fixed_ns + combine_ns;
       });
       if (t * 100 < best * 90) {
@@ -167,6 +190,7 @@ void order_backward(psa_plan_t* p, const std::vector<std::vector<int32_t>>& tile
         part->bwd_split = split;
       }
     }
+    if (part->bwd_split > 1) ctas.swap(sorted);
   }
   part->cta0 = int32_t(p->bwd_cta_map.size() / 2);
   part->n_ctas = int32_t(ctas.size());
