@@ -297,25 +297,31 @@ PyObject* rope(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // plan(cu, prefix, chosen, rejected, n_q_heads, n_kv_heads, head_dim, scale) -> (handle, tokens, pairs, live tiles, partial
 // tiles, workspace bytes), a status code (not 0), or None.  The arrays are int32 buffers, contiguous and one-dimensional.
 PyObject* plan(PyObject*, PyObject* const* a, Py_ssize_t n) {
-  int64_t v[3];
-  float scale;
-  if (n != 8 || !g_ready || !take_float(a[7], &scale)) return none();
-  for (int i = 0; i < 3; ++i)
-    if (!take_int(a[4 + i], &v[i]) || v[i] < INT32_MIN || v[i] > INT32_MAX) return none();
-  Py_buffer b[4];
-  int held = 0;
-  bool ok = true;
-  for (; held < 4 && ok; ++held) {
-    if (PyObject_GetBuffer(a[held], &b[held], PyBUF_C_CONTIGUOUS | PyBUF_FORMAT) != 0) {
-      PyErr_Clear();
-      ok = false;
-      break;
+  return guarded([&]() -> PyObject* {
+    int64_t v[3];
+    float scale;
+    if (n != 8 || !g_ready || !take_float(a[7], &scale)) return none();
+    for (int i = 0; i < 3; ++i)
+      if (!take_int(a[4 + i], &v[i]) || v[i] < INT32_MIN || v[i] > INT32_MAX) return none();
+    struct Buffers {
+      Py_buffer b[4];
+      int held = 0;
+      ~Buffers() {
+        while (held > 0) PyBuffer_Release(&b[--held]);
+      }
+    } buffers;
+    const Py_buffer* b = buffers.b;
+    for (int i = 0; i < 4; ++i) {
+      if (PyObject_GetBuffer(a[i], &buffers.b[i], PyBUF_C_CONTIGUOUS | PyBUF_FORMAT) != 0) {
+        PyErr_Clear();
+        return none();
+      }
+      buffers.held = i + 1;
+      if (b[i].ndim != 1 || b[i].itemsize != 4 || !b[i].format || b[i].format[0] != 'i' || b[i].format[1]) return none();
     }
-    ok = b[held].ndim == 1 && b[held].itemsize == 4 && b[held].format && b[held].format[0] == 'i' && !b[held].format[1];
-  }
-  PyObject* result = nullptr;
-  if (ok && b[1].shape[0] < INT32_MAX && b[0].shape[0] == b[1].shape[0] + 1 && b[2].shape[0] == b[1].shape[0] &&
-      b[3].shape[0] == b[1].shape[0]) {
+    if (b[1].shape[0] >= INT32_MAX || b[0].shape[0] != b[1].shape[0] + 1 || b[2].shape[0] != b[1].shape[0] ||
+        b[3].shape[0] != b[1].shape[0])
+      return none();
     psa_plan_t* p = nullptr;
     int64_t T = 0, pairs = 0, live = 0, partial = 0;
     size_t ws = 0;
@@ -326,12 +332,10 @@ PyObject* plan(PyObject*, PyObject* const* a, Py_ssize_t n) {
                                            int32_t(b[1].shape[0]), int32_t(v[0]), int32_t(v[1]), int32_t(v[2]), scale, 0, st, &p);
       return made == PSA_OK ? g_lib.stats(p, &T, &pairs, &live, &partial, &ws) : made;
     });
-    result = rc == PSA_OK ? Py_BuildValue("(NLLLLn)", PyLong_FromVoidPtr(p), (long long)T, (long long)pairs, (long long)live,
-                                          (long long)partial, Py_ssize_t(ws))
-                          : PyLong_FromLong(rc);
-  }
-  while (held > 0) PyBuffer_Release(&b[--held]);
-  return result ? result : none();
+    return rc == PSA_OK ? Py_BuildValue("(NLLLLn)", PyLong_FromVoidPtr(p), (long long)T, (long long)pairs, (long long)live,
+                                        (long long)partial, Py_ssize_t(ws))
+                        : PyLong_FromLong(rc);
+  });
 }
 
 // destroy(handle)
