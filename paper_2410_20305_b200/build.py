@@ -10,7 +10,6 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libpsa.so")
 LIB_DEBUG = os.path.join(HERE, "libpsa_debug.so")   # the same sources with -DPSA_DEBUG_BOUNDS (checked global indices)
-NATIVE = os.path.join(HERE, "psa_native.so")
 SOURCES = ["psa_plan.cpp", "psa_host_helpers.cpp", "psa_api.cu", "psa_fwd.cu", "psa_bwd.cu", "psa_bwd_static.cu", "psa_selftest.cu",
            "dpo_logp.cu", "dpo_loss.cu", "psa_rope.cu"]
 
@@ -45,29 +44,48 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
     return lib
 
 
-def build_native(force: bool = False) -> str:
-    """Builds psa_native.so, the compiled route of the binding's calls (csrc/psa_native.cpp), against the torch that runs."""
-    source = os.path.join(CSRC, "psa_native.cpp")
-    deps = [source, os.path.join(ROOT, "include", "psa.h")]
-    if not force and os.path.exists(NATIVE) and all(os.path.getmtime(d) <= os.path.getmtime(NATIVE) for d in deps):
-        return NATIVE
+def native_path() -> str:
+    """Where psa_native's library for this interpreter and this torch lies.  It has torch's tensor layout and CPython's
+    ABI compiled in, so one that was built for others must never be loaded: they are part of its name."""
     import sysconfig
     import torch
-    home = os.path.dirname(torch.__file__)
-    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
-    include = [os.path.join(ROOT, "include"), os.path.join(home, "include"),
-               os.path.join(home, "include", "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"],
-               os.path.join(cuda, "include")]
-    # into place at once: another process may be about to load it
-    out = "%s.%d.tmp" % (NATIVE, os.getpid())
-    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI]
-    cmd += [a for d in include for a in ("-I", d)] + ["-o", out, source, "-L", os.path.join(home, "lib")]
-    cmd += ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if res.returncode != 0:
-        raise RuntimeError("g++ failed building psa_native.so: " + res.stderr[-2000:])
-    os.replace(out, NATIVE)
-    return NATIVE
+    torch_tag = "".join(c if c.isalnum() or c in ".+" else "_" for c in torch.__version__)
+    return os.path.join(HERE, "psa_native.torch-%s-abi%d%s" % (torch_tag, torch._C._GLIBCXX_USE_CXX11_ABI,
+                                                             sysconfig.get_config_var("EXT_SUFFIX")))
+
+
+def build_native(force: bool = False) -> str:
+    """Builds the compiled route of the binding's calls (csrc/psa_native.cpp) against the torch that runs."""
+    source, native = os.path.join(CSRC, "psa_native.cpp"), native_path()
+    deps = [source, os.path.join(ROOT, "include", "psa.h")]
+
+    def current():
+        return os.path.exists(native) and all(os.path.getmtime(d) <= os.path.getmtime(native) for d in deps)
+
+    if not force and current():
+        return native
+    import fcntl
+    import sysconfig
+    import torch
+    with open(source) as lock:   # one process of a node builds, the others wait for it
+        fcntl.flock(lock, fcntl.LOCK_EX)
+        if not force and current():
+            return native
+        home = os.path.dirname(torch.__file__)
+        cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+        include = [os.path.join(ROOT, "include"), os.path.join(home, "include"),
+                   os.path.join(home, "include", "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"],
+                   os.path.join(cuda, "include")]
+        # into place at once: another process may be about to load it
+        out = "%s.%d.tmp" % (native, os.getpid())
+        cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI]
+        cmd += [a for d in include for a in ("-I", d)] + ["-o", out, source, "-L", os.path.join(home, "lib")]
+        cmd += ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+        res = subprocess.run(cmd, capture_output=True, text=True)
+        if res.returncode != 0:
+            raise RuntimeError("g++ failed building psa_native: " + res.stderr[-2000:])
+        os.replace(out, native)
+    return native
 
 
 if __name__ == "__main__":

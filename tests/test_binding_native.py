@@ -4,6 +4,10 @@ import os
 import subprocess
 import sys
 
+import pytest
+
+from paper_2410_20305_b200 import build
+
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
@@ -24,3 +28,18 @@ B.load_library()
 a = lambda *x: np.array(x, dtype=np.int32)
 print(B._native.plan(a(0, 10), a(4), a(3), a(3), 4, 2, 64, 0.0))
 """).split() == ["None"]
+
+
+@pytest.mark.parametrize("other", [("torch.__version__", "99.1.0+cu1"), ("torch._C._GLIBCXX_USE_CXX11_ABI", 7)])
+def test_a_library_of_another_torch_or_interpreter_is_not_taken(monkeypatch, other):
+    import sysconfig
+    here = build.build_native()
+    assert os.path.exists(here) and build.build_native() == here
+    monkeypatch.setattr(other[0], other[1])
+    elsewhere = build.native_path()
+    assert elsewhere != here and not os.path.exists(elsewhere)
+    monkeypatch.undo()
+    suffix = sysconfig.get_config_var("EXT_SUFFIX")
+    assert here.endswith(suffix)   # the interpreter's ABI and platform
+    monkeypatch.setattr(sysconfig, "get_config_var", lambda name: ".cpython-399" + suffix if name == "EXT_SUFFIX" else None)
+    assert build.native_path() not in (here, elsewhere)
