@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import sys
 
 import numpy as np
 
@@ -43,6 +44,8 @@ def load_library():
     debug library (libpsa_debug.so: the same code with checked global indices) is loaded instead."""
     global _lib
     if _lib is not None:
+        if not _native_tried and _cuda_ready():
+            _load_native()
         return _lib
     from . import build as _build
     debug = os.environ.get("PSA_DEBUG_LIB", "") not in ("", "0")
@@ -93,20 +96,25 @@ def load_library():
         elif name != "psa_status_string":
             getattr(lib, name).restype = C.c_int
     _lib = lib
-    _load_native(lib, _build)
-    return lib
+    return load_library()
 
 
 # The compiled route of the calls below (csrc/psa_native.cpp), or None.  It takes a call on the current stream whose
-# arguments are as they have to be, and returns None for any other, which then goes on here.
+# arguments are as they have to be, and returns None for any other, which then goes on here.  It is loaded, and built
+# where it has to be, by the first call of a process that uses CUDA: packing, labels and host-only plans need neither
+# torch nor a compiler.
 _native = None
+_native_tried = False
 _NATIVE_ENTRIES = ("psa_fwd", "psa_bwd", "psa_bwd_f32", "dpo_logp_f64sum", "dpo_logp_bwd", "dpo_loss", "simpo_loss",
                    "orpo_loss", "psa_rope", "psa_plan", "psa_plan_stats", "psa_plan_destroy")
 
 
-def _load_native(lib, build):
-    global _native
+def _load_native():
+    global _native, _native_tried
+    _native_tried = True
     try:
+        from . import build
+        lib = load_library()
         import torch  # noqa: F401  (its libraries have to be there before the extension's)
         from importlib.machinery import ExtensionFileLoader
         from importlib.util import module_from_spec, spec_from_loader
@@ -119,10 +127,17 @@ def _load_native(lib, build):
         _native = None
 
 
+def _cuda_ready():
+    """True where torch's CUDA context exists already (which imports nothing and creates none)."""
+    torch = sys.modules.get("torch")
+    cuda = getattr(torch, "cuda", None)
+    return cuda is not None and cuda.is_initialized()
+
+
 def _fast(stream):
     """The compiled route, where the call is on the current stream and `load_library` is the one above."""
-    if stream is None and load_library is _load_library:
-        return _native if _lib is not None else (load_library() and _native)
+    if stream is None and load_library is _load_library and load_library():
+        return _native
     return None
 
 
@@ -206,11 +221,6 @@ def _want_attention(plan, bf16, f32=(), lse=None, cuda=True):
             _want(t, name, (T, heads[kind], d), torch.float32, cuda, placement)
         if lse is not None:
             _want(lse, "lse", (plan.n_q_heads, T), torch.float32, cuda, placement)
-
-
-def _cuda_ready():
-    import torch
-    return torch.cuda.is_initialized()
 
 
 class Plan:

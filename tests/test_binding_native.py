@@ -24,7 +24,7 @@ def test_plan_without_a_device_is_left_to_the_binding():
     assert _python("""
 import numpy as np
 from paper_2410_20305_b200 import binding as B
-B.load_library()
+B._load_native()
 a = lambda *x: np.array(x, dtype=np.int32)
 print(B._native.plan(a(0, 10), a(4), a(3), a(3), 4, 2, 64, 0.0))
 """).split() == ["None"]
@@ -43,3 +43,18 @@ def test_a_library_of_another_torch_or_interpreter_is_not_taken(monkeypatch, oth
     assert here.endswith(suffix)   # the interpreter's ABI and platform
     monkeypatch.setattr(sysconfig, "get_config_var", lambda name: ".cpython-399" + suffix if name == "EXT_SUFFIX" else None)
     assert build.native_path() not in (here, elsewhere)
+
+
+def test_calls_on_the_host_alone_need_neither_torch_nor_a_compiler():
+    assert _python("""
+import sys, subprocess
+from paper_2410_20305_b200 import binding as B
+B.load_library()
+subprocess.run = None      # nothing is built from here on
+B.psa_pack_ffd([5, 7, 3], 10)
+B.psa_pack_ffd_emit([5, 7], [1, 1], [1, 1], 20)
+B.psa_logp_labels(range(9), [0, 9], [3], [3], [3])
+B.psa_position_ids([0, 9], [3], [3], [3])
+B.psa_plan([0, 9], [3], [3], [3], 4, 2, 64, host_only=True).close()
+print("torch" in sys.modules, B._native, B._native_tried)
+""").split() == ["False", "None", "False"]
