@@ -58,3 +58,19 @@ B.psa_position_ids([0, 9], [3], [3], [3])
 B.psa_plan([0, 9], [3], [3], [3], 4, 2, 64, host_only=True).close()
 print("torch" in sys.modules, B._native, B._native_tried)
 """).split() == ["False", "None", "False"]
+
+
+def test_a_route_that_cannot_be_had_is_said_once_and_the_calls_go_on():
+    assert _python("""
+import warnings
+from paper_2410_20305_b200 import binding as B, build
+def fails():
+    raise RuntimeError("no compiler here")
+build.build_native = fails
+B._cuda_ready = lambda: True
+with warnings.catch_warnings(record=True) as said:
+    warnings.simplefilter("always")
+    for _ in range(3):
+        B.psa_pack_ffd([5, 7, 3], 10)
+print(len(said), "no compiler here" in str(said[0].message), said[0].category.__name__, B._native)
+""").split() == ["1", "True", "RuntimeWarning", "None"]
