@@ -100,9 +100,10 @@ def load_library():
 
 
 # The compiled route of the calls below (csrc/psa_native.cpp), or None.  It takes a call on the current stream whose
-# arguments are as they have to be, and returns None for any other, which then goes on here.  It is loaded, and built
-# where it has to be, by the first call of a process that uses CUDA: packing, labels and host-only plans need neither
-# torch nor a compiler.
+# arguments are as they have to be, and returns None for any other, which then goes on here.  It is asked where a call has
+# no stream=, and buffers as a training step passes them: psa_bwd and psa_bwd_f32 with workspace=, dpo_logp_bwd with
+# dlogits=, psa_rope with out=, dpo_logp without out= and scratch=.  It is loaded, and built where it has to be, by the
+# first call of a process that uses CUDA: packing, labels and host-only plans need neither torch nor a compiler.
 _native = None
 _native_tried = False
 _NATIVE_ENTRIES = ("psa_fwd", "psa_bwd", "psa_bwd_f32", "dpo_logp_f64sum", "dpo_logp_bwd", "dpo_loss", "simpo_loss",
@@ -138,8 +139,8 @@ def _cuda_ready():
 
 
 def _fast(stream):
-    """The compiled route, where the call is on the current stream and `load_library` is the one above."""
-    if stream is None and load_library is _load_library and load_library():
+    """The compiled route, where the call is on the current stream."""
+    if stream is None and load_library():
         return _native
     return None
 
@@ -153,9 +154,6 @@ def _i32(a):
     if type(a) is np.ndarray and a.dtype == np.int32 and a.flags.c_contiguous:
         return a
     return np.ascontiguousarray(np.asarray(a, dtype=np.int32))
-
-
-_load_library = load_library   # (`load_library` itself may be replaced, for instance to write calls down)
 
 
 # Pointers and streams are handed over as plain integers (every such argument is declared c_void_p).

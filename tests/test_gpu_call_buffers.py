@@ -122,3 +122,32 @@ def test_backward_workspace_on_a_stream_that_is_not_current(monkeypatch, name, a
     assert torch.equal(grads[1], want[1]) and torch.equal(grads[2], want[2])
     # dq: unordered fp32 adds, rounded to bf16
     assert max_abs(grads[0], want[0].cpu().double().numpy()) <= 0.0625
+
+
+@pytest.mark.parametrize("compiled", [True, False])
+def test_what_a_call_allocates_belongs_to_the_current_stream(monkeypatch, compiled):
+    """Sums, log-probs, loss and coefficients of a call while a side stream is current: what the main stream allocates and
+    writes meanwhile shares no memory with them."""
+    args, want = _logp_inputs(300, 1024, 6, 6)
+    assert B.load_library() and B._native is not None
+    if not compiled:
+        monkeypatch.setattr(B, "_native", None)
+    ref = torch.zeros(6, device="cuda")
+    side = torch.cuda.Stream()
+    a = torch.randn((4096, 4096), device="cuda", dtype=torch.bfloat16)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        for _ in range(40):
+            a @ a                                      # the side stream is busy while the calls return
+        got = B.dpo_logp(*args)
+        loss, coef = B.dpo_loss(got, ref, 0.1)
+    held = [torch.full((n,), float("nan"), dtype=t, device="cuda") for n in (1, 6, 7) for t in (torch.float32, torch.float64)
+            for _ in range(16)]
+    torch.cuda.current_stream().synchronize()
+    side.synchronize()
+    assert np.abs(got.cpu().double().numpy() - want).max() <= 1e-4 * np.abs(want).max()
+    # (of the log-probs as they came: fp32 differences of values of up to 500 times 0.1, 2^-23 500 0.1 = 6e-6 in the exponent)
+    want_loss, want_coef = orc.dpo_loss(got.cpu().double().numpy(), np.zeros(6), 0.1)
+    assert abs(loss.item() - want_loss) <= 1e-4 * abs(want_loss)
+    assert np.abs(coef.cpu().double().numpy() - want_coef).max() <= 1e-4 * np.abs(want_coef).max()
+    assert all(t.isnan().all() for t in held)
