@@ -512,14 +512,18 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       if (e_cur & 2) iteration(it, std::true_type{});
       else iteration(it, std::false_type{});
     }
-    // dV is final before the last dK and dQ are: without a cluster it leaves while these run (7965 tokens, 16 heads of
-    // 64: 126 -> 124 us; at 128 0.2 % of short packs).
-    if constexpr (kSplit) mbar_wait(bar(B_DONE), 0, wctx);
-    else mbar_wait(bar(B_DO_EMPTY), (n_it - 1) & 1, wctx);
+    // dV is final before the last dK and dQ are: at head size 64, without a cluster, it leaves while these run (7965 tokens,
+    // 16 heads of 64: 128.9 -> 126.7 us).  Not at 128, where that gains nothing on short lists (7727 tokens, 32/8 heads, 233.9
+    // and 235.0) and the kernel is slower on long ones (one sample of 12000, 32/8: 2967 -> 3029; of 16700, 8/2: 1474 -> 1516).
+    constexpr bool kDvFirst = D == 64 && !kSplit;
+    if constexpr (kDvFirst) mbar_wait(bar(B_DO_EMPTY), (n_it - 1) & 1, wctx);
+    else mbar_wait(bar(B_DONE), 0, wctx);
     tc_fence_after();
     auto before_dk = [&]() {
-      mbar_wait(bar(B_DONE), 0, wctx);
-      tc_fence_after();
+      if constexpr (kDvFirst) {
+        mbar_wait(bar(B_DONE), 0, wctx);
+        tc_fence_after();
+      }
     };
 
     // ---- epilogue: this half's columns of dV and dK (scaled) -> bf16, or fp32 as they are
@@ -648,10 +652,23 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                          pack_bf16x2(__uint_as_float(v[8 * i + 6]) * mul, __uint_as_float(v[8 * i + 7]) * mul));
           }
         }
+        if constexpr (kDvFirst) {
+          fence_proxy_async_smem();
+          named_bar_sync(1, 256);
+          if (leader) {
+            for (int s = 0; s < L::kSub; ++s) tma_store_3d(which ? &tm_dk : &tm_dv, tile + s * L::kSubBytes, s * 64, hk, rec.row0);
+            tma_commit_group();
+          }
+        }
+      }
+      if constexpr (!kDvFirst) {
         fence_proxy_async_smem();
         named_bar_sync(1, 256);
         if (leader) {
-          for (int s = 0; s < L::kSub; ++s) tma_store_3d(which ? &tm_dk : &tm_dv, tile + s * L::kSubBytes, s * 64, hk, rec.row0);
+          for (int s = 0; s < L::kSub; ++s) {
+            tma_store_3d(&tm_dv, sV + s * L::kSubBytes, s * 64, hk, rec.row0);
+            tma_store_3d(&tm_dk, sK + s * L::kSubBytes, s * 64, hk, rec.row0);
+          }
           tma_commit_group();
         }
       }
