@@ -93,7 +93,8 @@ enum {
 
 // kSplit: the iterations of one (key tile, kv head) are shared by the CTAs of a cluster, rank r taking the r-th
 // part of them; dV and dK are summed over the cluster through distributed shared memory before they leave.
-template <int D, bool kSplit>
+// kLate: when the workers touch the next iteration's statistics (see load_stat).
+template <int D, bool kSplit, bool kLate>
 __global__ void __launch_bounds__(kBwdThreads, 1)
 psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do,
@@ -317,20 +318,26 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     const float cl = prm.scale_log2;
 
     // Per-column statistics of an iteration's query tile: workers 0..127 fetch lse, workers 128..255 fetch delta, each
-    // for column (wt & 127).  They are asked for an iteration ahead and first touched (scaled, stored) at its end: with
-    // the scaling beside the load, and divisions to find the next query head and list position, the workers stood still
-    // for 1200 of an iteration's 3600 clocks at head size 64.  us of the backward: 20774 tokens, 16 heads of 64, 500 ->
-    // 471; 7965 tokens, 16 of 64, fp32 gradients, 131 -> 126; 7727 tokens, 32/8 of 128, 221 -> 215; long lists at 128
-    // are paced by the other roles (31041 tokens 2435 -> 2424, one sample of 16700 1413 -> 1430).
+    // for column (wt & 127), and are asked for an iteration ahead.  Late, they are first touched (scaled, stored) at the
+    // iteration's end, and the query head and list position are counted: with the scaling beside the load, and divisions
+    // for the position, the workers stand still for 1200 of an iteration's 3600 clocks at head size 64.  us of the backward,
+    // early / late: 16700 tokens, 8/2 heads of 64, 1027 / 971; 7965 tokens, 16 of 64, fp32 gradients, 133 / 127; 7727 tokens,
+    // 32/8 of 128, 238 / 234; 16215, 32/8 of 128, 901 / 894.  Long lists at 128 are paced by the other roles, and early is the
+    // better one there (kLongLists has the figures).  Early, only the half of the workers whose load is scaled stands still;
+    // with the scaling taken out of the branch both halves do, and all of it is lost (one sample of 16700, 8/2 heads of 128:
+    // 1441 us early, 1454 late, 1534 early with both halves).
     const float* const stat_of = wt < 128 ? prm.lse : prm.delta;
     const float stat_mul = wt < 128 ? kLog2e : 1.f;
     auto load_stat = [&](int h, int e) {
       const int64_t qrow = int64_t(rec.ds) + (e >> 2) * kTile + (wt & 127), idx = int64_t(h) * prm.T + qrow;
       float x = 0.f;
-      if (qrow < prm.row_end && PSA_IN_BOUNDS(idx, int64_t(prm.Hq) * prm.T, prm.status)) x = stat_of[idx];
+      if (qrow < prm.row_end && PSA_IN_BOUNDS(idx, int64_t(prm.Hq) * prm.T, prm.status)) {
+        if constexpr (kLate) x = stat_of[idx];
+        else x = wt < 128 ? prm.lse[idx] * kLog2e : prm.delta[idx];
+      }
       return x;
     };
-    auto store_stat = [&](int st, float x) { (wt < 128 ? s_lse : s_delta)[st * kTile + (wt & 127)] = x * stat_mul; };
+    auto store_stat = [&](int st, float x) { (wt < 128 ? s_lse : s_delta)[st * kTile + (wt & 127)] = kLate ? x * stat_mul : x; };
     // Query head, list position and entry of the current iteration.
     int h_cur = 0, li_cur = 0, e_cur = 0;
     if (!kSplit || n_it > 0) {
@@ -349,16 +356,20 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     auto iteration = [&](int it, auto precise_tag) {
       constexpr bool kPrecise = decltype(precise_tag)::value;
       const int st = it & 1;
-      const int e = e_cur;
+      const int e = kLate ? e_cur : entry_of(it);
       const int q0 = (e >> 2) * kTile;
       float next_stat = 0.f;
       if (it + 1 < n_it) {
-        if (++li_cur == n_list) {
-          li_cur = 0;
-          ++h_cur;
+        if constexpr (kLate) {
+          if (++li_cur == n_list) {
+            li_cur = 0;
+            ++h_cur;
+          }
+          e_cur = entry_at(li_cur);
+          next_stat = load_stat(h_cur, e_cur);
+        } else {
+          next_stat = load_stat(head_of(it + 1), entry_of(it + 1));
         }
-        e_cur = entry_at(li_cur);
-        next_stat = load_stat(h_cur, e_cur);
       }
 
       mbar_wait(bar(B_S_FULL), it & 1, wctx);
@@ -509,7 +520,7 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       named_bar_sync(1, 256);
     };
     for (int it = 0; it < n_it; ++it) {
-      if (e_cur & 2) iteration(it, std::true_type{});
+      if ((kLate ? e_cur : entry_of(it)) & 2) iteration(it, std::true_type{});
       else iteration(it, std::false_type{});
     }
     // dV is final before the last dK and dQ are: at head size 64, without a cluster, it leaves while these run (7965 tokens,
@@ -900,7 +911,10 @@ psa_status_t launch_bwd_t(const psa_plan_t* plan, const PlanPart& part, const vo
       !make_tile_map_bf16(&tm_dk, dk, rows, plan->Hkv, D) || !make_tile_map_bf16(&tm_dv, dv, rows, plan->Hkv, D))
     return PSA_ERR_CUDA;
   const int split = part.bwd_split;
-  auto kernel = split > 1 ? psa_bwd_kernel<D, true> : psa_bwd_kernel<D, false>;
+  auto kernel = split > 1 ? psa_bwd_kernel<D, true, true> : psa_bwd_kernel<D, false, true>;
+  if constexpr (D == 128) {
+    if (split == 1 && part.bwd_long_lists) kernel = psa_bwd_kernel<D, false, false>;
+  }
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kRequest) != cudaSuccess)
     return PSA_ERR_CUDA;
 

@@ -36,6 +36,13 @@ struct FewKeyRow {
 };
 static_assert(sizeof(FewKeyRow) == 16, "FewKeyRow is 4 int32");
 
+// Where the backward's lists count as long: the mean list, weighted by its work, of one sample of 64 tiles.  us of the
+// backward at head size 128, statistics touched early / late (psa_bwd.cu):
+//   one sample, 32/8 heads: 6000 tokens (32 tiles) 814 / 815, 9000 (48) 1716 / 1722, 12000 (63) 2931 / 2954, 16700 (88) 5524 / 5542
+//   one sample of 16700, 8/2 heads (88) 1441 / 1454, of 9000, 8/8 (48) 437 / 439, of 16000, 8/8 (84) 1277 / 1293
+//   packs of 7 to 11 samples, 32/8 heads: 31041 tokens (20) 2453 / 2442, 15154 (13) 946 / 941, 16215 (12) 897 / 884
+constexpr int kLongLists = 43;
+
 // The part of a plan that one launch covers: the whole pack, or a run of whole samples of it (psa_step_host overlaps
 // the copies of one run with the kernels of another).  Offsets index the plan's device arrays.
 struct PlanPart {
@@ -44,6 +51,7 @@ struct PlanPart {
   int32_t cta0 = 0, n_ctas = 0;          // (key tile, kv head) pairs of the backward's launch order
   int32_t few0 = 0, n_few = 0;           // few-key rows
   int32_t fwd_items_per_cta = 2;         // work items (query tile, query head) that a CTA of the forward takes: 1 or 2
+  int32_t bwd_long_lists = 0;            // the backward's lists, weighted by their work, are kLongLists tiles or longer
   int32_t bwd_split = 1;                 // CTAs (a cluster) that share the iterations of one such pair: 1, 2, 4 or 8
 };
 

@@ -107,13 +107,15 @@ void order_backward(psa_plan_t* p, const std::vector<std::vector<int32_t>>& tile
   std::iota(order.begin(), order.end(), s0);
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return work[a - s0] > work[b - s0]; });
   Order grouped;
-  int64_t total_work = 0;
+  int64_t total_work = 0, squares = 0;
   for (int s : order)
     for (int hk = 0; hk < p->Hkv; ++hk)
       for (int32_t t : tiles_of[s]) {
         grouped.emplace_back(t, hk);
         total_work += p->kv_tiles[t].list_cnt;
+        squares += int64_t(p->kv_tiles[t].list_cnt) * p->kv_tiles[t].list_cnt;
       }
+  part->bwd_long_lists = total_work > 0 && squares >= kLongLists * total_work;
   // Makespan of an order on `slots` slots, a pair with a list of n taking cost(n).
   std::vector<int64_t> free_at;
   auto makespan = [&](const Order& o, size_t slots, auto cost) {
