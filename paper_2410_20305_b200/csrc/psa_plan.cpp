@@ -83,6 +83,51 @@ void items_per_cta(const psa_plan_t* p, int n_sm, PlanPart* part) {
   part->fwd_items_per_cta = work * 100 >= 94 * 2 * int64_t(n_sm) * two_longest ? 2 : 1;
 }
 
+// List scheduling on `n` slots: every pair goes to the slot that is free first.
+struct Slots {
+  std::vector<int64_t> free_at;   // a heap, earliest first
+  std::vector<int64_t> scratch;
+  int64_t end = 0;                // when the last pair so far ends
+  bool sorted = true;             // free_at ascends as a whole
+
+  explicit Slots(size_t n = 0) : free_at(n, 0) {}
+
+  void take(int64_t cost) {
+    const size_t n = free_at.size();
+    const int64_t t = free_at[0] + cost;   // the earliest slot takes the pair and sinks to its new place
+    end = std::max(end, t);
+    size_t i = 0;
+    for (size_t k = 1; k < n; k = 2 * i + 1) {
+      if (k + 1 < n && free_at[k + 1] < free_at[k]) ++k;
+      if (free_at[k] >= t) break;
+      free_at[i] = free_at[k];
+      i = k;
+    }
+    free_at[i] = t;
+    sorted = false;
+  }
+
+  // `count` pairs of one cost.  Many at a time: the slots that are taken ascend, and so do their new times, so that the next
+  // one is the smaller head of two ascending rows.
+  void take_equal(int32_t count, int64_t cost) {
+    if (count < 32) {
+      for (; count > 0; --count) take(cost);
+      return;
+    }
+    if (!sorted) std::sort(free_at.begin(), free_at.end());
+    sorted = true;
+    const size_t n = free_at.size();
+    scratch.resize(size_t(count) + n);
+    int64_t* const taken = scratch.data();
+    size_t i = 0, j = 0;
+    for (size_t k = 0; k < size_t(count); ++k)
+      taken[k] = cost + (i < n && (j == k || free_at[i] <= taken[j]) ? free_at[i++] : taken[j++]);
+    end = std::max(end, taken[count - 1]);
+    std::merge(free_at.begin() + i, free_at.end(), taken + j, taken + count, taken + count);
+    std::copy(taken + count, taken + count + n, free_at.begin());
+  }
+};
+
 // Launch order of the backward for the samples [s0, s1), appended to the plan's list, and the number of CTAs that share
 // the iterations of one (key tile, kv head) pair.
 //
@@ -97,75 +142,84 @@ void items_per_cta(const psa_plan_t* p, int n_sm, PlanPart* part) {
 //   19431, 32/8 of 128 (8)    1039 / 1031 / 1015 / 1028 / 1046 / 1107     16215, 32/8 of 128 (7)  892 / 893 / 871 / 850 / 864 / 930
 //   7727, 32/8 of 128 (3.7)   226 / 224 / 223 / 218 / 211 / 227           accumulators of 19 to 42 MB:
 //   4952, 8/8 of 128 (2.2)    109 / 110 / 106 / 101 / 96 / 91             5465, 32/8 of 64 (2.4)  223 / 222 / 217 / 204 / 191 / 166
+//
+// The simulation costs no more than the order is worth to a step that plans for itself (psa_plan and psa_plan_destroy on
+// the host, us: 7965 tokens, 16/16 heads of 64, 242 -> 50; 31041, 32/8 of 128, 290 -> 154): the shares have the grouped order's start in
+// common, which is simulated once, and a sorted end is runs of equal pairs; sorting and simulating the order for each share
+// was the difference.
 void order_backward(psa_plan_t* p, const std::vector<std::vector<int32_t>>& tiles_of, int s0, int s1, int n_sm,
                     PlanPart* part) {
-  typedef std::vector<std::pair<int32_t, int32_t>> Order;   // (key tile record, kv head)
+  struct Pair {
+    int32_t tile, kv_head, len;   // key tile record, kv head, length of the tile's list
+  };
   std::vector<int64_t> work(s1 - s0, 0);
-  for (int s = s0; s < s1; ++s)
+  size_t n_pairs = 0;
+  for (int s = s0; s < s1; ++s) {
     for (int32_t t : tiles_of[s]) work[s - s0] += p->kv_tiles[t].list_cnt;
+    n_pairs += tiles_of[s].size() * size_t(p->Hkv);
+  }
   std::vector<int> order(s1 - s0);
   std::iota(order.begin(), order.end(), s0);
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return work[a - s0] > work[b - s0]; });
-  Order grouped;
+  std::vector<Pair> pairs;   // grouped, until the end of this function
+  pairs.reserve(n_pairs);
   int64_t total_work = 0, squares = 0;
+  int32_t longest = 0;
   for (int s : order)
     for (int hk = 0; hk < p->Hkv; ++hk)
       for (int32_t t : tiles_of[s]) {
-        grouped.emplace_back(t, hk);
-        total_work += p->kv_tiles[t].list_cnt;
-        squares += int64_t(p->kv_tiles[t].list_cnt) * p->kv_tiles[t].list_cnt;
+        const int32_t n = p->kv_tiles[t].list_cnt;
+        pairs.push_back(Pair{t, hk, n});
+        total_work += n;
+        squares += int64_t(n) * n;
+        longest = std::max(longest, n);
       }
   part->bwd_long_lists = total_work > 0 && squares >= kLongLists * total_work;
-  // Makespan of an order on `slots` slots, a pair with a list of n taking cost(n).
-  std::vector<int64_t> free_at;
-  auto makespan = [&](const Order& o, size_t slots, auto cost) {
-    int64_t end = 0;
-    if (o.size() <= slots) {
-      for (const auto& c : o) end = std::max(end, cost(p->kv_tiles[c.first].list_cnt));
-      return end;
-    }
-    free_at.assign(slots, 0);   // a heap, earliest first: the earliest slot takes the pair and sinks to its new place
-    for (const auto& c : o) {
-      const int64_t t = free_at[0] + cost(p->kv_tiles[c.first].list_cnt);
-      end = std::max(end, t);
-      size_t i = 0;
-      for (size_t k = 1; k < slots; k = 2 * i + 1) {
-        if (k + 1 < slots && free_at[k + 1] < free_at[k]) ++k;
-        if (free_at[k] >= t) break;
-        free_at[i] = free_at[k];
-        i = k;
-      }
-      free_at[i] = t;
-    }
-    return end;
-  };
   const int64_t iter_ns = p->d == 128 ? 2050 : 1600, fixed_ns = p->d == 128 ? 8000 : 7000, combine_ns = 3000;
   const int64_t group = p->Hq / p->Hkv;
   auto alone = [&](int32_t n) { return n * group * iter_ns + fixed_ns; };
-  // The pairs with the last `permille` of the work longest first.
-  auto tail_sorted = [&](int64_t permille) {
-    Order o = grouped;
+
+  // First pair of the longest-first end that holds the last `permille` of the work.
+  auto end_of = [&](int64_t permille) {
     int64_t acc = 0;
     size_t at = 0;
-    while (at < o.size() && acc * 1000 < total_work * (1000 - permille)) acc += p->kv_tiles[o[at++].first].list_cnt;
-    std::stable_sort(o.begin() + at, o.end(), [&](const auto& a, const auto& b) {
-      return p->kv_tiles[a.first].list_cnt > p->kv_tiles[b.first].list_cnt;
-    });
-    return o;
+    while (at < pairs.size() && acc * 1000 < total_work * (1000 - permille)) acc += pairs[at++].len;
+    return at;
   };
-  Order ctas = grouped;
-  int64_t best = makespan(ctas, n_sm, alone);
-  if (part == &p->whole && grouped.size() > size_t(n_sm)) {
+  size_t sorted_from = pairs.size();
+  int64_t best = 0;
+  const bool whole = part == &p->whole;
+  if (pairs.size() <= size_t(n_sm)) {
+    best = alone(longest);
+  } else if (whole) {
+    // Candidates: first pairs of the sorted ends, in the order in which they are preferred.
+    size_t candidates[4], n_candidates = 0;
     const bool in_l2 = int64_t(p->T) * p->Hq * p->d * 4 <= (int64_t(64) << 20);
-    const int64_t wave = std::min<int64_t>(1000, 1150 * int64_t(n_sm) / int64_t(grouped.size()));
+    const int64_t wave = std::min<int64_t>(1000, 1150 * int64_t(n_sm) / int64_t(pairs.size()));
+    candidates[n_candidates++] = end_of(wave);
+    if (in_l2)
+      for (int64_t permille : {300, 500, 1000}) candidates[n_candidates++] = end_of(permille);
+    // One pass over the grouped order, which stops at every candidate's start to keep the slots as they are there.
+    Slots slots(n_sm), at_start[4];
+    for (size_t i = 0; i < pairs.size(); ++i) {
+      for (size_t c = 0; c < n_candidates; ++c)
+        if (candidates[c] == i) at_start[c] = slots;
+      slots.take(alone(pairs[i].len));
+    }
+    best = slots.end;
+    // No order is shorter than the mean load or the longest pair.
+    const int64_t least = std::max((total_work * group * iter_ns + int64_t(pairs.size()) * fixed_ns) / n_sm, alone(longest));
     int64_t shortest = best * 985 / 1000;
-    for (int64_t permille : {wave, int64_t(300), int64_t(500), int64_t(1000)}) {
-      if (permille != wave && !in_l2) break;
-      Order o = tail_sorted(permille);
-      const int64_t t = makespan(o, n_sm, alone);
+    std::vector<int32_t> of_length(longest + 1);
+    for (size_t c = 0; c < n_candidates && least < shortest; ++c) {
+      if (candidates[c] == pairs.size()) continue;
+      std::fill(of_length.begin(), of_length.end(), 0);
+      for (size_t i = candidates[c]; i < pairs.size(); ++i) ++of_length[pairs[i].len];
+      for (int32_t n = longest; n > 0; --n) at_start[c].take_equal(of_length[n], alone(n));
+      const int64_t t = at_start[c].end;
       if (t >= shortest) continue;
       shortest = best = t;
-      ctas.swap(o);
+      sorted_from = candidates[c];
     }
   }
   // CTAs per pair: where the pairs are few, the longest of them lasts longer than the rest of the chip is busy.  Sharing
@@ -176,34 +230,40 @@ void order_backward(psa_plan_t* p, const std::vector<std::vector<int32_t>>& tile
   //   16700 tokens, 8/2 heads of 128 (262)          1383 / 1262 / 1374 / 1482 in short runs, 1376 / 1389 in long ones,
   //   where the power limit sets the clock: a prediction of less than 10 % is not worth it.
   //   5061 tokens, 32/8 heads of 128 (328)          264 / 270 / 354 / 575
-  if (part != &p->whole) {
+  if (!whole) {
     part->bwd_split = p->whole.bwd_split;   // dk and dv are summed in the same order, and come out the same, as for the whole
-  } else if (ctas.size() <= 2 * size_t(n_sm)) {
+  } else if (pairs.size() <= 2 * size_t(n_sm)) {
     // Pairs that share their iterations are few, and handed out longest first as a whole (2008 tokens, 32/8 heads of 128,
     // 145 -> 103 us; 2436 tokens, 32/8 of 64, 151 -> 110).  Where only that order makes it worth while, lists of less than
     // 20 iterations have to gain a quarter: they have more fixed costs than the simulation knows of.
-    int64_t longest = 0;
-    for (const auto& c : grouped) longest = std::max<int64_t>(longest, p->kv_tiles[c.first].list_cnt * group);
-    const int64_t need = longest >= 20 ? 90 : 75;
-    Order sorted = tail_sorted(1000);
+    const int64_t need = longest * group >= 20 ? 90 : 75;
+    std::vector<int32_t> of_length(longest + 1, 0);
+    for (const Pair& c : pairs) ++of_length[c.len];
     for (int split : {2, 4, 8}) {
-      const size_t slots = split == 2 ? n_sm / 2 : (split == 4 ? n_sm * 33 / 148 : n_sm * 15 / 148);
+      const size_t n_slots = std::max(1, split == 2 ? n_sm / 2 : (split == 4 ? n_sm * 33 / 148 : n_sm * 15 / 148));
       auto shared = [&](int32_t n) { return (n * group + split - 1) / split * iter_ns + fixed_ns + combine_ns; };
-      const int64_t t = makespan(grouped, std::max<size_t>(slots, 1), shared);
-      const int64_t t_sorted = makespan(sorted, std::max<size_t>(slots, 1), shared);
-      if (t * 100 < best * 90 || t_sorted * 100 < best * need) {
-        best = std::min(t, t_sorted);
+      int64_t grouped = shared(longest), sorted = grouped;
+      if (pairs.size() > n_slots) {
+        Slots in_turn(n_slots), longest_first(n_slots);
+        for (const Pair& c : pairs) in_turn.take(shared(c.len));
+        for (int32_t n = longest; n > 0; --n) longest_first.take_equal(of_length[n], shared(n));
+        grouped = in_turn.end;
+        sorted = longest_first.end;
+      }
+      if (grouped * 100 < best * 90 || sorted * 100 < best * need) {
+        best = std::min(grouped, sorted);
         part->bwd_split = split;
       }
     }
-    if (part->bwd_split > 1) ctas.swap(sorted);
+    if (part->bwd_split > 1) sorted_from = 0;
   }
   part->cta0 = int32_t(p->bwd_cta_map.size() / 2);
-  part->n_ctas = int32_t(ctas.size());
-  p->bwd_cta_map.reserve(p->bwd_cta_map.size() + ctas.size() * 2);
-  for (const auto& c : ctas) {
-    p->bwd_cta_map.push_back(c.first);
-    p->bwd_cta_map.push_back(c.second);
+  part->n_ctas = int32_t(pairs.size());
+  std::stable_sort(pairs.begin() + sorted_from, pairs.end(), [](const Pair& a, const Pair& b) { return a.len > b.len; });
+  p->bwd_cta_map.reserve(p->bwd_cta_map.size() + pairs.size() * 2);
+  for (const Pair& c : pairs) {
+    p->bwd_cta_map.push_back(c.tile);
+    p->bwd_cta_map.push_back(c.kv_head);
   }
 }
 
