@@ -224,6 +224,29 @@ def _want_attention(plan, bf16, f32=(), lse=None, cuda=True):
             _want(lse, "lse", (plan.n_q_heads, T), torch.float32, cuda, placement)
 
 
+def _want_flat(t, name, dtype, n):
+    """Raises ValueError unless `t` is a contiguous CUDA tensor of this dtype with at least n elements."""
+    if not t.is_cuda or t.dtype != dtype or not t.is_contiguous() or t.numel() < n:
+        raise ValueError("%s: a contiguous CUDA tensor of at least %d %s is needed" % (name, n, dtype))
+
+
+def _want_status(status):
+    """Raises ValueError unless a status word is one that kernels can add to (an empty tensor is none, as None is)."""
+    if status is None:
+        return
+    size = status.numel() * status.element_size()
+    if not status.is_cuda or 0 < size < 4 or status.data_ptr() % 4:
+        raise ValueError("status: an int32 CUDA tensor is needed")
+
+
+def _want_room(t, name, n):
+    """Raises ValueError unless CUDA tensor `t` has n bytes, in its shape and in the memory behind it (an expanded tensor
+    has fewer than its shape says)."""
+    size = t.element_size()
+    if not t.is_cuda or min(t.numel() * size, t.untyped_storage().nbytes() - t.storage_offset() * size) < n:
+        raise ValueError("%s: a CUDA buffer of at least %d bytes is needed" % (name, n))
+
+
 class Plan:
     """Owner of a psa_plan_t*.  One plan serves every layer of a step."""
 
@@ -316,6 +339,7 @@ def psa_fwd(plan: Plan, q, k, v, o=None, lse=None, status=None, stream=None):
             _check("psa_fwd", code)
             return o, lse
     _want_attention(plan, [("q", q, "q"), ("k", k, "kv"), ("v", v, "kv"), ("o", o, "q")], lse=lse)
+    _want_status(status)
     _check("psa_fwd", load_library().psa_fwd(plan._h, _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse), _ptr(status),
                                              _stream(stream)))
     return o, lse
@@ -340,8 +364,8 @@ def psa_bwd(plan: Plan, d_o, q, k, v, o, lse, dq=None, dk=None, dv=None, workspa
                            ("dq", dq, "q"), ("dk", dk, "kv"), ("dv", dv, "kv")], lse=lse)
     if workspace is None:
         workspace = _temporary(max(plan.bwd_workspace_bytes, 256), torch.uint8, q.device, stream)
-    if not workspace.is_cuda or workspace.numel() * workspace.element_size() < plan.bwd_workspace_bytes:
-        raise ValueError("workspace: a CUDA buffer of at least %d bytes is needed" % plan.bwd_workspace_bytes)
+    _want_room(workspace, "workspace", plan.bwd_workspace_bytes)
+    _want_status(status)
     _check("psa_bwd", load_library().psa_bwd(plan._h, _ptr(d_o), _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse),
                                              _ptr(dq), _ptr(dk), _ptr(dv), _ptr(workspace), _ptr(status),
                                              _stream(stream)))
@@ -366,8 +390,8 @@ def psa_bwd_f32(plan: Plan, d_o, q, k, v, o, lse, dq=None, dk=None, dv=None, wor
                     f32=[("dq", dq, "q"), ("dk", dk, "kv"), ("dv", dv, "kv")], lse=lse)
     if workspace is None:
         workspace = _temporary(max(plan.bwd_workspace_bytes, 256), torch.uint8, q.device, stream)
-    if not workspace.is_cuda or workspace.numel() * workspace.element_size() < plan.bwd_workspace_bytes:
-        raise ValueError("workspace: a CUDA buffer of at least %d bytes is needed" % plan.bwd_workspace_bytes)
+    _want_room(workspace, "workspace", plan.bwd_workspace_bytes)
+    _want_status(status)
     _check("psa_bwd_f32", load_library().psa_bwd_f32(plan._h, _ptr(d_o), _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse),
                                                      _ptr(dq), _ptr(dk), _ptr(dv), _ptr(workspace), _ptr(status),
                                                      _stream(stream)))
@@ -423,8 +447,10 @@ def dpo_logp(logits, targets, segment_ids, n_segments, fork_rows=None, fork_targ
         out = torch.empty(n_segments, dtype=torch.float32, device=logits.device)
     if scratch is None:
         scratch = _temporary(max(n_segments, 0) + 1, torch.float64, logits.device, stream)
-    elif not scratch.is_cuda or scratch.numel() * scratch.element_size() < 8 * (n_segments + 1):
-        raise ValueError("scratch: a CUDA buffer of at least %d bytes is needed" % (8 * (n_segments + 1)))
+    else:
+        _want_room(scratch, "scratch", 8 * (n_segments + 1))
+    _want_flat(out, "out", torch.float32, n_segments)
+    _want_status(status)
     _check("dpo_logp", load_library().dpo_logp_f64sum(
         _ptr(logits), dt, n_rows, vocab, logits.stride(0) if n_rows > 1 else vocab, _ptr(targets), _ptr(segment_ids),
         _ptr(fork_rows), _ptr(fork_targets), _ptr(fork_segments), n_forks, n_segments, _ptr(out), _ptr(scratch),
@@ -454,6 +480,7 @@ def psa_bwd_static_scratch(plan: Plan, d_o, q, k, v, o, lse, dq, dk, dv, status=
     PsaError (status 3).  Calls that overlap on the GPU share the array and must be serialised."""
     _want_attention(plan, [("d_o", d_o, "q"), ("q", q, "q"), ("k", k, "kv"), ("v", v, "kv"), ("o", o, "q"),
                            ("dq", dq, "q"), ("dk", dk, "kv"), ("dv", dv, "kv")], lse=lse)
+    _want_status(status)
     _check("psa_bwd_static_scratch",
            load_library().psa_bwd_static_scratch(plan._h, _ptr(d_o), _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse),
                                                  _ptr(dq), _ptr(dk), _ptr(dv), _ptr(status), _stream(stream)))
@@ -476,6 +503,7 @@ def psa_step_host(plan: Plan, h_q, h_k, h_v, h_do, h_o, h_lse, h_dq, h_dk, h_dv,
                     lse=h_lse, cuda=False)
     if not (arena.is_cuda and arena.dtype == torch.uint8 and arena.is_contiguous()):
         raise ValueError("arena must be a contiguous uint8 CUDA tensor")
+    _want_status(status)
     _check("psa_step_host",
            load_library().psa_step_host(plan._h, _ptr(h_q), _ptr(h_k), _ptr(h_v), _ptr(h_do), _ptr(h_o), _ptr(h_lse),
                                         _ptr(h_dq), _ptr(h_dk), _ptr(h_dv), _ptr(arena),
@@ -495,6 +523,7 @@ def dpo_loss(policy_logps, ref_logps, beta, stream=None):
     import torch
     assert policy_logps.is_cuda and policy_logps.dtype == torch.float32 and policy_logps.is_contiguous()
     assert ref_logps.shape == policy_logps.shape and ref_logps.dtype == torch.float32 and ref_logps.is_contiguous()
+    _want_flat(ref_logps, "ref_logps", torch.float32, policy_logps.numel())
     n = policy_logps.numel() // 2
     loss = torch.empty(1, dtype=torch.float32, device=policy_logps.device)
     coef = torch.empty(2 * n, dtype=torch.float32, device=policy_logps.device)
@@ -516,6 +545,8 @@ def simpo_loss(policy_logps, lengths, beta, gamma, status=None, stream=None):
     import torch
     assert policy_logps.is_cuda and policy_logps.dtype == torch.float32 and policy_logps.is_contiguous()
     assert lengths.is_cuda and lengths.dtype == torch.int32 and lengths.shape == policy_logps.shape
+    _want_flat(lengths, "lengths", torch.int32, policy_logps.numel())
+    _want_status(status)
     n = policy_logps.numel() // 2
     loss = torch.empty(1, dtype=torch.float32, device=policy_logps.device)
     coef = torch.empty(2 * n, dtype=torch.float32, device=policy_logps.device)
@@ -538,6 +569,8 @@ def orpo_loss(policy_logps, lengths, lam, status=None, stream=None):
     import torch
     assert policy_logps.is_cuda and policy_logps.dtype == torch.float32 and policy_logps.is_contiguous()
     assert lengths.is_cuda and lengths.dtype == torch.int32 and lengths.shape == policy_logps.shape
+    _want_flat(lengths, "lengths", torch.int32, policy_logps.numel())
+    _want_status(status)
     n = policy_logps.numel() // 2
     loss = torch.empty(1, dtype=torch.float32, device=policy_logps.device)
     coef = torch.empty(2 * n, dtype=torch.float32, device=policy_logps.device)
@@ -567,6 +600,14 @@ def dpo_logp_bwd(logits, targets, segment_ids, coef, fork_rows=None, fork_target
     if dlogits is None:
         dlogits = torch.empty_strided(logits.shape, logits.stride(), dtype=logits.dtype, device=logits.device)
     assert dlogits.dtype == logits.dtype and dlogits.stride() == logits.stride()
+    if not dlogits.is_cuda or dlogits.shape[0] < n_rows or dlogits.shape[1] < vocab:
+        raise ValueError("dlogits: a CUDA tensor of the logits' shape is needed")
+    for t, name in ((targets, "targets"), (segment_ids, "segment_ids")):
+        _want_flat(t, name, torch.int32, n_rows)
+    for t, name in ((fork_rows, "fork_rows"), (fork_targets, "fork_targets"), (fork_segments, "fork_segments")):
+        if t is not None:
+            _want_flat(t, name, torch.int32, n_forks)
+    _want_status(status)
     _check("dpo_logp_bwd", load_library().dpo_logp_bwd(
         _ptr(logits), dt, n_rows, vocab, logits.stride(0) if n_rows > 1 else vocab, _ptr(targets), _ptr(segment_ids),
         _ptr(fork_rows), _ptr(fork_targets), _ptr(fork_segments), n_forks, int(coef.numel()), _ptr(coef),
@@ -652,6 +693,7 @@ def psa_rope(x, position_ids, rope_theta=10000.0, out=None, stream=None):
     assert position_ids.is_cuda and position_ids.dtype == torch.int32 and position_ids.numel() == x.shape[0]
     if out is None:
         out = torch.empty_like(x)
+    _want_flat(out, "out", torch.bfloat16, x.numel())
     _check("psa_rope", load_library().psa_rope(_ptr(x), _ptr(out), _ptr(position_ids), x.shape[0], x.shape[1],
                                               x.shape[2], float(rope_theta), _stream(stream)))
     return out

@@ -63,8 +63,9 @@ bool take_status(PyObject* o, void** p) {
   *p = nullptr;
   if (o == Py_None) return true;
   const at::Tensor* t = plain(o);
-  if (t) *p = t->data_ptr();
-  return t != nullptr;
+  if (!t || (t->numel() > 0 && t->nbytes() < 4)) return false;
+  *p = t->data_ptr();
+  return reinterpret_cast<uintptr_t>(*p) % 4 == 0;
 }
 bool take_int(PyObject* o, int64_t* v) {
   if (!PyLong_CheckExact(o)) return false;
@@ -155,7 +156,9 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         !take3(a[9], g, p.T, p.Hkv, p.d, &dk) || !take3(a[10], g, p.T, p.Hkv, p.d, &dv) || !take_status(a[12], &st))
       return none();
     const at::Tensor* ws = plain(a[11]);
-    if (!ws || ws->numel() * ws->element_size() < p.ws) return none();
+    if (!ws || int64_t(ws->nbytes()) < p.ws ||
+        int64_t(ws->storage().nbytes()) - ws->storage_offset() * int64_t(ws->itemsize()) < p.ws)
+      return none();
     const float* l = static_cast<const float*>(lse);
     int32_t* s = static_cast<int32_t*>(st);
     void *const w = ws->data_ptr(), *const on = stream();

@@ -110,6 +110,35 @@ def test_both_routes_refuse_the_same_calls(monkeypatch):
         B.psa_fwd(plan, q, k, v, o=o, lse=lse)
 
 
+def test_both_routes_refuse_buffers_that_are_too_small_or_elsewhere(monkeypatch):
+    pack, (q, k, v, d_o), logits, (targets, segments, *forks), lengths = _inputs(5, 2, 150, (4, 2, 64), torch.bfloat16, 256)
+    plan = device_plan(pack)
+    o, lse = B.psa_fwd(plan, q, k, v)
+    ws = torch.empty(plan.bwd_workspace_bytes, dtype=torch.uint8, device="cuda")
+    g = [torch.empty_like(t) for t in (q, k, v)]
+    lp, d = torch.zeros(2 * pack.n_samples, device="cuda"), torch.empty_like(logits)
+    byte = torch.zeros(8, dtype=torch.uint8, device="cuda")
+    bwd = lambda t=targets, s=segments, f=forks, to=d, status=None: B.dpo_logp_bwd(logits, t, s, lp, *f, dlogits=to, status=status)
+    calls = [
+        lambda: bwd(t=targets.long()), lambda: bwd(t=targets[:-1]), lambda: bwd(s=segments.cpu()), lambda: bwd(s=segments[:-1]),
+        lambda: bwd(f=[forks[0], forks[1][:-1], forks[2]]), lambda: bwd(f=[forks[0], forks[1], forks[2].long()]),
+        lambda: bwd(to=d[:-1]), lambda: bwd(to=torch.empty(d.shape, dtype=d.dtype)),
+        lambda: B.psa_rope(q, targets, out=torch.empty_like(q)[:-1]), lambda: B.psa_rope(q, targets, out=torch.empty_like(q).cpu()),
+        lambda: B.dpo_loss(lp, lp.cpu(), 0.1), lambda: B.simpo_loss(lp, lengths.cpu(), 0.1, 0.2),
+        lambda: B.psa_bwd(plan, d_o, q, k, v, o, lse, *g, workspace=byte[:1].clone().expand(ws.numel())),
+    ]
+    for status in (torch.zeros(1, dtype=torch.int32), byte[:1], byte[1:5]):
+        calls += [lambda s=status: bwd(status=s), lambda s=status: B.psa_fwd(plan, q, k, v, status=s),
+                  lambda s=status: B.dpo_logp(logits, targets, segments, 2 * pack.n_samples, status=s),
+                  lambda s=status: B.psa_bwd(plan, d_o, q, k, v, o, lse, *g, workspace=ws, status=s),
+                  lambda s=status: B.simpo_loss(lp, lengths, 0.1, 0.2, status=s), lambda s=status: B.orpo_loss(lp, lengths, 0.1, status=s)]
+    for route in (B._native, None):
+        monkeypatch.setattr(B, "_native", route)
+        for call in calls:
+            with pytest.raises((ValueError, AssertionError)):
+                call()
+
+
 @pytest.mark.parametrize("seed,n,longest,heads", [(1, 1, 130, (4, 4, 64)), (2, 2, 400, (8, 2, 128)), (4, 3, 90, (4, 2, 64))])
 def test_launches_behind_one_another_see_what_came_before(seed, n, longest, heads):
     """Inputs and labels are rewritten on the stream right before every step, and the same buffers are used again."""
