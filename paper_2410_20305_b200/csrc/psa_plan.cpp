@@ -234,8 +234,13 @@ void order_backward(psa_plan_t* p, const std::vector<std::vector<int32_t>>& tile
     part->bwd_split = p->whole.bwd_split;   // dk and dv are summed in the same order, and come out the same, as for the whole
   } else if (pairs.size() <= 2 * size_t(n_sm)) {
     // Pairs that share their iterations are few, and handed out longest first as a whole (2008 tokens, 32/8 heads of 128,
-    // 145 -> 103 us; 2436 tokens, 32/8 of 64, 151 -> 110).  Where only that order makes it worth while, lists of less than
-    // 20 iterations have to gain a quarter: they have more fixed costs than the simulation knows of.
+    // 145 -> 103 us; 2436 tokens, 32/8 of 64, 151 -> 110), also where the simulation has the grouped order 2 % shorter (1429
+    // tokens, 32/8 of 128, 82.4 against 86.5; 2299, 32/8 of 64, 65.6 against 69.2).  What sharing takes is judged by the
+    // shorter of the two simulated times, although one order is launched: by the launched order's alone four CTAs become two
+    // in 73 of 40000 packs, which takes 0.96 to 1.25 times as long, 1.08 in the middle (4400 tokens, 8/2 of 64, 59 -> 70).
+    // Where only the sorted order makes sharing worth while, lists of less than 20 iterations have to gain a quarter, which
+    // errs on the side of one CTA per pair: of 518 packs of up to 296 pairs the choice differs from 10 % throughout on two
+    // (1375 tokens, 32/8 of 128, 69.6 us with one CTA, 51.3 with two; 1682 tokens, 8/8 of 128, 45.3 and 39.0).
     const int64_t need = longest * group >= 20 ? 90 : 75;
     std::vector<int32_t> of_length(longest + 1, 0);
     for (const Pair& c : pairs) ++of_length[c.len];

@@ -131,6 +131,9 @@ def _rule(pack, tiles):
 
 def _packs():
     yield wl.config_pack(0)
+    # clusters for which the grouped order is the shorter one in the simulation
+    yield wl.pack_from_lengths("turn-a", [(29, 141, 19), (2, 21, 13), (292, 82, 38), (173, 50, 18), (251, 41, 84), (427, 132, 103)], 32, 8, 128)
+    yield wl.pack_from_lengths("turn-b", [(745, 43, 198), (550, 32, 183), (126, 35, 45), (121, 139, 119)], 32, 8, 64)
     yield wl.pack_from_lengths("empty", [(0, 0, 0)], 4, 2, 64)
     for heads in ((32, 8, 128), (16, 16, 64), (8, 2, 128), (8, 2, 64), (32, 8, 64), (8, 8, 128)):
         for seed, (n, longest) in enumerate([(1, 900), (2, 2500), (5, 700), (9, 1500), (30, 200), (12, 60)]):
