@@ -84,7 +84,7 @@ struct MaxSum {
 };
 
 // One block; n_samples is small.
-__global__ void dpo_loss_kernel(const float* __restrict__ pol, const float* __restrict__ ref, int n, float beta,
+__global__ void dpo_loss_kernel(const float* pol, const float* ref, int n, float beta,
                                 float* __restrict__ loss, float* __restrict__ coef) {
   __shared__ float part[32];
   behind_wait();
@@ -108,7 +108,7 @@ __global__ void dpo_loss_kernel(const float* __restrict__ pol, const float* __re
 }
 
 // Length-normalised, reference-free variant (SimPO); one block.
-__global__ void simpo_loss_kernel(const float* __restrict__ pol, const int32_t* __restrict__ len, int n, float beta,
+__global__ void simpo_loss_kernel(const float* pol, const int32_t* len, int n, float beta,
                                   float gamma, float* __restrict__ loss, float* __restrict__ coef,
                                   int32_t* __restrict__ status) {
   __shared__ float part[32];
@@ -140,7 +140,7 @@ __global__ void simpo_loss_kernel(const float* __restrict__ pol, const int32_t* 
 }
 
 // Odds-ratio variant (ORPO); one block.
-__global__ void orpo_loss_kernel(const float* __restrict__ pol, const int32_t* __restrict__ len, int n, float lam,
+__global__ void orpo_loss_kernel(const float* pol, const int32_t* len, int n, float lam,
                                  float* __restrict__ loss, float* __restrict__ coef, int32_t* __restrict__ status) {
   __shared__ float part[32];
   behind_wait();
@@ -276,10 +276,9 @@ __device__ __forceinline__ float block_lse2(MaxSum acc, float2* s_part /* [kThre
 // between their sweeps, loaded with an evict-last policy in the first and evict-first in the second.
 template <typename T, int kThreads, bool kStaged, int kPerSm>
 __global__ void __launch_bounds__(kThreads, kPerSm)
-dpo_logp_bwd_kernel(const T* __restrict__ logits, int64_t vocab, int64_t row_stride, const int32_t* __restrict__ targets,
-                    const int32_t* __restrict__ segment_ids, const int32_t* __restrict__ fork_rows,
-                    const int32_t* __restrict__ fork_targets, const int32_t* __restrict__ fork_segments,
-                    int32_t n_forks, int32_t n_segments, const float* __restrict__ coef, T* __restrict__ dlogits,
+dpo_logp_bwd_kernel(const T* logits, int64_t vocab, int64_t row_stride, const int32_t* targets, const int32_t* segment_ids,
+                    const int32_t* fork_rows, const int32_t* fork_targets, const int32_t* fork_segments,
+                    int32_t n_forks, int32_t n_segments, const float* coef, T* __restrict__ dlogits,
                     int32_t* __restrict__ status) {
   constexpr int E = Elem<T>::kVec;
   constexpr int kParts = 4;

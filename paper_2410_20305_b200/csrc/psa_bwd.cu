@@ -784,7 +784,7 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 // clears the fp32 dq accumulator (same element mapping), which saves a separate pass over it.
 template <int D>
 __global__ void __launch_bounds__(256)
-psa_bwd_delta_kernel(const __nv_bfloat16* __restrict__ d_o, const __nv_bfloat16* __restrict__ o,
+psa_bwd_delta_kernel(const __nv_bfloat16* d_o, const __nv_bfloat16* o,
                      float* __restrict__ delta, float* __restrict__ dq_accum, int64_t row0,
                      int64_t row1 /* of T*Hq */, int32_t T, int32_t Hq, int32_t* status) {
   constexpr int kLanes = D / 8;  // threads per (t, h) row
@@ -867,7 +867,7 @@ psa_bwd_delta_few_keys_kernel(const FewKeyRow* __restrict__ rows, const __nv_bfl
 // dq = bf16(dq_accum).  Four independent 16-byte loads in flight per thread and streaming (evict-first)
 // accesses: the pass runs at the copy bandwidth (one load per thread left it 20 % short of it).
 __global__ void __launch_bounds__(256)
-psa_bwd_convert_kernel(const float4* __restrict__ acc, uint2* __restrict__ dq, int64_t n_vec4) {
+psa_bwd_convert_kernel(const float4* acc, uint2* __restrict__ dq, int64_t n_vec4) {
   const int64_t base = (int64_t(blockIdx.x) * blockDim.x) * 4 + threadIdx.x;
   behind_wait();
   behind_go();
