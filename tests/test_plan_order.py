@@ -152,3 +152,20 @@ def test_order_and_split_follow_the_rules(reader, pack):
         assert got == (order if (row0, row1) == (0, pack.total_tokens) else grouped), k
         n = [tiles[i][1] for i, _ in grouped]
         assert bool(long) == (sum(x * x for x in n) >= 43 * sum(n) > 0)
+
+
+@pytest.mark.parametrize("lengths,heads,split,kept", [
+    ([(3000, 300, 301), (900, 200, 252)], (8, 8, 128), 1, "less than half"),
+    ([(2600, 500, 200), (1500, 300, 420), (300, 90, 77)], (32, 8, 128), 1, "about half"),
+    ([(1500, 300, 209)], (32, 8, 128), 2, "none"),
+    ([(700, 130, 60), (1, 0, 1), (250, 129, 128)], (16, 16, 64), 1, "none")])
+def test_packs_of_the_gradient_test_take_the_orders_that_they_are_there_for(reader, lengths, heads, split, kept):
+    """How much of the grouped order is left at the start (tests/test_gpu_bwd_order.py)."""
+    pack = wl.pack_from_lengths("order", lengths, *heads)
+    tiles, parts = _read(reader, pack)
+    grouped, got = _grouped(tiles, 0, pack.total_tokens, pack.n_kv_heads), parts[0][4]
+    same = next((i for i, (a, b) in enumerate(zip(grouped, got)) if a != b), len(got)) / len(got)
+    assert parts[0][2] == split
+    assert {"about half": 0.4 < same < 0.6, "less than half": same < 0.5, "none": same < 0.1}[kept], same
+    lists = [tiles[i][1] for i, _ in got[int(same * len(got)) + 1:]]
+    assert lists == sorted(lists, reverse=True)
