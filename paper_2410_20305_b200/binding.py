@@ -634,6 +634,8 @@ def psa_pack_ffd_emit(prefix_len, chosen_len, rejected_len, capacity, paired=Fal
     (P, C, 0), (P, R, 0) per unit.  Host only."""
     P, Cc, R = _i32(prefix_len), _i32(chosen_len), _i32(rejected_len)
     n = len(P)
+    if len(Cc) < n or len(R) < n:
+        raise ValueError("chosen_len and rejected_len must have an entry for every one of prefix_len")
     m = n * (2 if paired else 1)
     bins = np.zeros(max(n, 1), dtype=np.int32)
     off = np.zeros(n + 1, dtype=np.int32)
@@ -659,8 +661,8 @@ def psa_logp_labels(token_ids, cu_seqlens, prefix_len, chosen_len, rejected_len)
     tok, cu = _i32(token_ids), _i32(cu_seqlens)
     P, Cc, R = _i32(prefix_len), _i32(chosen_len), _i32(rejected_len)
     n, T = len(P), int(cu[-1])
-    if len(cu) != n + 1 or len(tok) < T:
-        raise ValueError("cu_seqlens must have n+1 entries and token_ids at least T entries")
+    if len(cu) != n + 1 or len(tok) < T or len(Cc) < n or len(R) < n:
+        raise ValueError("cu_seqlens must have n+1 entries, the length arrays n and token_ids at least T entries")
     targets, seg = np.zeros(max(T, 1), dtype=np.int32), np.zeros(max(T, 1), dtype=np.int32)
     fr, ft, fs = (np.zeros(max(n, 1), dtype=np.int32) for _ in range(3))
     nf = C.c_int32()
@@ -674,6 +676,9 @@ def psa_logp_labels(token_ids, cu_seqlens, prefix_len, chosen_len, rejected_len)
 def psa_position_ids(cu_seqlens, prefix_len, chosen_len, rejected_len):
     """Position ids int32 [T] of the shared layout: rejected tokens restart right after the prompt."""
     cu, P, Cc, R = _i32(cu_seqlens), _i32(prefix_len), _i32(chosen_len), _i32(rejected_len)
+    n = len(P)
+    if len(cu) < n + 1 or len(Cc) < n or len(R) < n or cu[-1] < cu[n]:
+        raise ValueError("cu_seqlens must have n+1 entries and the three length arrays n entries")
     out = np.zeros(max(int(cu[-1]), 1), dtype=np.int32)
     _check("psa_position_ids", load_library().psa_position_ids(cu.ctypes.data, P.ctypes.data, Cc.ctypes.data,
                                                               R.ctypes.data, len(P), out.ctypes.data))

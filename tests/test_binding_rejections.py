@@ -74,3 +74,17 @@ def test_device_status_word_maps_to_status_codes():
     assert B.psa_check_device_status(B.PSA_DEVSTAT_BAD_SEGMENT) == 6
     lib = B.load_library()
     assert lib.psa_selftest_wait_expiry(None, 1000, None, None) == 1     # refused before any launch
+
+
+@pytest.mark.parametrize("short", ["cu", "chosen", "rejected"])
+def test_host_calls_refuse_arrays_that_are_too_short(short):
+    a = {"cu": [0, 9, 18], "prefix": [3, 3], "chosen": [3, 3], "rejected": [3, 3]}
+    a[short] = a[short][:-1]
+    cu, *lengths = (np.array(x, dtype=np.int32) for x in a.values())
+    with pytest.raises(ValueError):
+        B.psa_position_ids(cu, *lengths)
+    with pytest.raises(ValueError):
+        B.psa_logp_labels(np.arange(18, dtype=np.int32), cu, *lengths)
+    if short != "cu":
+        with pytest.raises(ValueError):
+            B.psa_pack_ffd_emit(*lengths, capacity=40)
