@@ -1,9 +1,16 @@
-"""Thin ctypes binding of libpsa's C ABI (include/psa.h).
+"""Thin binding of libpsa's C ABI (include/psa.h).
 
 Argument marshalling only: every step of the path runs inside the library's
 CUDA kernels.  torch is used for device memory and streams.  There is no CPU
 fallback: if the shared library is missing or a call fails, an exception is
 raised.
+
+Calls go through ctypes, or, as a training step makes them, through a compiled
+route that takes 4 to 9 us less of the host: psa_plan, psa_fwd and the losses
+without stream=, psa_bwd and psa_bwd_f32 without stream= and with workspace=,
+dpo_logp without stream=, out= and scratch=, dpo_logp_bwd without stream= and
+with dlogits=, psa_rope without stream= and with out=.  Results and refusals
+are the same.
 """
 from __future__ import annotations
 
@@ -100,10 +107,9 @@ def load_library():
 
 
 # The compiled route of the calls below (csrc/psa_native.cpp), or None.  It takes a call on the current stream whose
-# arguments are as they have to be, and returns None for any other, which then goes on here.  It is asked where a call has
-# no stream=, and buffers as a training step passes them: psa_bwd and psa_bwd_f32 with workspace=, dpo_logp_bwd with
-# dlogits=, psa_rope with out=, dpo_logp without out= and scratch=.  It is loaded, and built where it has to be, by the
-# first call of a process that uses CUDA: packing, labels and host-only plans need neither torch nor a compiler.
+# arguments are as they have to be, and returns None for any other, which then goes on here.  It is loaded, and built
+# where it has to be, by the first call of a process that uses CUDA: packing, labels and host-only plans need neither torch
+# nor a compiler.
 _native = None
 _native_tried = False
 _NATIVE_ENTRIES = ("psa_fwd", "psa_bwd", "psa_bwd_f32", "dpo_logp_f64sum", "dpo_logp_bwd", "dpo_loss", "simpo_loss",
