@@ -524,8 +524,9 @@ psa_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       else iteration(it, std::false_type{});
     }
     // dV is final before the last dK and dQ are: at head size 64, without a cluster, it leaves while these run (7965 tokens,
-    // 16 heads of 64: 128.9 -> 126.7 us).  Not at 128, where that gains nothing on short lists (7727 tokens, 32/8 heads, 233.9
-    // and 235.0) and the kernel is slower on long ones (one sample of 12000, 32/8: 2967 -> 3029; of 16700, 8/2: 1474 -> 1516).
+    // 16 heads of 64: 128.9 -> 126.7 us).  Not at 128, where that gains 0.8 % on short lists without groups (8189 tokens, 8/8 heads,
+    // 169.1 -> 167.8), nothing with them (7727 tokens, 32/8, 233.9 and 235.0), and costs 2 % on longer ones (one sample of 6000
+    // tokens, 32/8: 804 -> 822; of 12000, 32/8: 2967 -> 3029; of 16700, 8/2: 1474 -> 1516).
     constexpr bool kDvFirst = D == 64 && !kSplit;
     if constexpr (kDvFirst) mbar_wait(bar(B_DO_EMPTY), (n_it - 1) & 1, wctx);
     else mbar_wait(bar(B_DONE), 0, wctx);
